@@ -413,7 +413,7 @@ void batch_query_desc(const tp_plan* p, const BatchPrep& x, void* join_slots, ui
     B.fast = x.fast ? 1 : 0;
     for (int t = 0; t < p->n_sum; ++t) {
         B.sum_mode[t] = x.smem ? x.mode[t] : 0;
-        B.sum_off[t] = x.smem ? x.bounds[t].lo : 0;
+        B.sum_off[t] = x.smem ? (int64_t)x.bounds[t].lo : 0;
     }
     if (x.join) {
         B.b.key.ptr = d.dim->dev_cols[d.join.dim_col];

@@ -1606,19 +1606,20 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
         const bool want_staged = !(e->cfg.flags & TP_FLAG_NO_STAGED);
         bool fast = want_staged && !(e->cfg.flags & TP_FLAG_EXACT_ONLY) && sums_fit_int64(p, S.fact);
         tpk::TermBounds bounds[tpk::MAX_SUM] = {};
-        if (fast) term_bounds(p, S.fact, bounds);
+        if (want_staged) term_bounds(p, S.fact, bounds);
         int narrow[tpk::MAX_SUM] = {};
         narrow_products(p, S.fact, narrow);
         const bool want_jit = want_staged && !(e->cfg.flags & TP_FLAG_NO_JIT);
         int mode = -1;  // 0 plain exact, 1 staged exact, 2 staged 64-bit
         auto shared_core = [&](const tpk::QueryDev& q, uint64_t rows) -> tp_status {
             tpk::StageLayout L;
-            bool can = want_staged && tpk::staged_layout_shared(q, p->key_bits, mode != 1 && fast, bounds, rows,
-                                                                e->num_sms, tpk::AOT_GEOM, tpk::ST_MAX_STAGES, &L);
+            bool can = want_staged &&
+                       tpk::staged_layout_shared(q, p->key_bits, mode != 1 && fast ? tpk::DW_FAST : tpk::DW_EXACT,
+                                                 bounds, rows, e->num_sms, tpk::AOT_GEOM, tpk::ST_MAX_STAGES, &L);
             if (mode < 0 && !can && fast) {  // no 32-bit table fits: exact staged table instead
                 fast = false;
-                can = want_staged && tpk::staged_layout_shared(q, p->key_bits, false, bounds, rows, e->num_sms,
-                                                               tpk::AOT_GEOM, tpk::ST_MAX_STAGES, &L);
+                can = want_staged && tpk::staged_layout_shared(q, p->key_bits, tpk::DW_EXACT, bounds, rows,
+                                                               e->num_sms, tpk::AOT_GEOM, tpk::ST_MAX_STAGES, &L);
             }
             if (mode < 0) mode = can ? (fast ? 2 : 1) : 0;
             if (mode == 2 && !can) return fail(TP_E_INTERNAL, "staged layout changed between batches");
@@ -1628,12 +1629,17 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
             if (mode > 0 && can) {
                 const void* jk = nullptr;
                 if (want_jit) {
+                    // sums that may leave int64 as 32-bit limbs: 64-bit shared
+                    // atomics only where the limbs' rows do not fit (or on request)
                     tpk::StageLayout LJ;
-                    if (tpk::staged_layout_shared(q, p->key_bits, mode == 2, bounds, rows, e->num_sms,
+                    const tpk::DenseWords dw = mode == 2                                 ? tpk::DW_FAST
+                                               : (e->cfg.flags & TP_FLAG_EXACT_ONLY) != 0 ? tpk::DW_EXACT
+                                                                                          : tpk::DW_WIDE;
+                    if (tpk::staged_layout_shared(q, p->key_bits, dw, bounds, rows, e->num_sms,
                                                   tpk::JIT_DENSE_GEOM, tpk::JIT_DENSE_STAGES, &LJ) &&
                         LJ.n_stages == tpk::JIT_DENSE_STAGES && rows >= (uint64_t)LJ.tile) {
                         std::string why;
-                        jk = jit_kernel(e, dense_shape(q, LJ, mode == 2, narrow), "tpj_dense", &why);
+                        jk = jit_kernel(e, dense_shape(q, LJ, dw, narrow), "tpj_dense", &why);
                         if (jk) {
                             L = LJ;   // the ahead-of-time kernel keeps its own layout
                             e->jit_launches++;
@@ -2098,7 +2104,7 @@ void narrow_products(const tp_plan* p, const tp_table* fact, int* out) {
 // compiled kernels (fields: jit_common.cuh).  mode[s]: 32-bit accumulation
 // mode of sum s (fast only).
 std::string shape_struct(const std::string& name, const tpk::QueryDev& q, const int8_t* mode_in, bool fast,
-                         bool lo_only, const int* narrow) {
+                         bool lo_only, const int* narrow, bool wide) {
     auto arr = [](const char* nm, const int* v, int n) {
         std::string r = std::string(nm) + "[" + std::to_string(n) + "] = {";
         for (int i = 0; i < n; ++i) r += (i ? ", " : "") + std::to_string(v[i]);
@@ -2144,13 +2150,14 @@ std::string shape_struct(const std::string& name, const tpk::QueryDev& q, const 
          ", " + arr("btype", btype, tpk::MAX_SUM) + ", " + arr("mode", mode, tpk::MAX_SUM) + ", " +
          arr("narrow", nar, tpk::MAX_SUM) + ";\n";
     r += std::string("    static constexpr bool fast = ") + (fast ? "true" : "false") +
-         ", lo_only = " + (!fast && lo_only ? "true" : "false") + ";\n};\n";
+         ", lo_only = " + (!fast && lo_only ? "true" : "false") + ", wide = " + (wide ? "true" : "false") + ";\n};\n";
     return r;
 }
 
 // The source of a dense staged launch's run-time compiled kernel.
-std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, bool fast, const int* narrow) {
-    return shape_struct("JS", q, L.sum_mode, fast, false, narrow) + "#include \"jit_dense.cuh\"\n";
+std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, tpk::DenseWords kind, const int* narrow) {
+    return shape_struct("JS", q, L.sum_mode, kind != tpk::DW_EXACT, false, narrow, kind == tpk::DW_WIDE) +
+           "#include \"jit_dense.cuh\"\n";
 }
 
 // Per-row term range of every sum slot, from column statistics.
@@ -2171,9 +2178,8 @@ void term_bounds(const tp_plan* p, const tp_table* fact, tpk::TermBounds* out) {
                 hi = c[i] > hi ? c[i] : hi;
             }
         }
-        // only used when sums_fit_int64 holds, so both ends fit in int64
-        out[s].lo = (int64_t)lo;
-        out[s].span = (uint64_t)(hi - lo);
+        out[s].lo = lo;   // within +-2^127: |a| <= 2^63, |k - b| < 2^64
+        out[s].span = (unsigned __int128)hi - (unsigned __int128)lo;
     }
 }
 

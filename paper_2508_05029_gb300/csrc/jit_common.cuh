@@ -20,11 +20,16 @@
 //   many                     the first join fans out (repeated build keys)
 //   ng, gside[], gtype[], gbits[]   group fields, first field highest
 //   ns, skind[], atype[], btype[]   sums: S_SUM / S_MUL_SUB and column types
-//   mode[]                   1: low word, 2: low + carry word (fast), 0: exact
+//   mode[]                   words a sum takes in the 32-bit table (fast): 1 low
+//                            word, 2 low + carry word, 3 or 4 limbs of an exact
+//                            sum; 0: exact 64-bit table
 //   narrow[]                 mode 2 MUL_SUB operands proved to fit in int32
-//   fast                     32-bit dense table (column bounds proved every
-//                            sum stays inside int64); otherwise the table holds
-//                            count[G], lo[s][G], hi[s][G] 64-bit words
+//   fast                     dense table of 32-bit words; otherwise the table
+//                            holds count[G], lo[s][G], hi[s][G] 64-bit words
+//   wide                     (fast, may be absent = false) sums may leave int64:
+//                            folded into both words of the 128-bit accumulators.
+//                            Without it the column bounds proved every sum stays
+//                            inside int64 and only low words are folded
 //   lo_only                  (not fast) sums proved to stay inside int64: add
 //                            64-bit terms to the low words only (the high words
 //                            are their sign extension); otherwise exact 128-bit
@@ -120,6 +125,30 @@ __device__ __forceinline__ constexpr uint32_t sum_word() {
     return w;
 }
 
+template <class...>
+struct MakeVoid { typedef void type; };
+template <class S, class = void>
+struct WideOf { static constexpr bool value = false; };
+template <class S>
+struct WideOf<S, typename MakeVoid<decltype(S::wide)>::type> { static constexpr bool value = S::wide; };
+
+// Adds the K limbs of w to K consecutive blocks of G 32-bit words, the carry
+// out of each limb (from the value its atomic returned) going to the next;
+// limbs beyond w's take carries only.  Exact modulo 2^(32 K).
+template <int K, int W>
+__device__ __forceinline__ void add_limbs(uint32_t* p, uint32_t G, const uint32_t (&w)[W]) {
+    uint32_t carry = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const uint64_t v = (uint64_t)(i < W ? w[i < W ? i : 0] : 0u) + carry;
+        carry = (uint32_t)(v >> 32);
+        if ((uint32_t)v != 0) {
+            const uint32_t old = atomicAdd(p + (uint64_t)i * G, (uint32_t)v);
+            carry += old + (uint32_t)v < old ? 1u : 0u;
+        }
+    }
+}
+
 // Group field F (compile-time recursion over the fields).
 template <class S, int F, class C>
 __device__ __forceinline__ void group_fields(const QueryDev& q, const C& c, uint32_t r0,
@@ -171,6 +200,32 @@ __device__ __forceinline__ void sums(const QueryDev& q, const Tab& t, const C& c
                 uint32_t v = c.template ld_lo<TA, CI_A + I>(r0, j);
                 if constexpr (MS) v *= k - c.template ld_lo<TB, CI_B + I>(r0, j);
                 if (pm >> j & 1u) atomicAdd(lo + g[j], v - off);
+            }
+        } else if constexpr (S::fast && S::mode[I] >= 3) {
+            // exact sums as 32-bit limbs: 32-bit shared-memory atomics are
+            // native where 64-bit ones are compare-and-swap loops.  Three
+            // limbs hold (term - offset) < 2^64 of up to 2^32 rows (the low
+            // 64 bits of a * (k - b) - off are exact); four hold any term
+            // modulo 2^128.  A fan-out query of 20M rows x 3 partners with one
+            // three-limb sum: 1.80 ms with 64-bit words, 1.34 ms with limbs.
+            uint32_t* p = (uint32_t*)t.base + (uint64_t)sum_word<S, I>() * t.G;
+#pragma unroll
+            for (int j = 0; j < ST_RPL; ++j) {
+                if (!(pm >> j & 1u)) continue;
+                const int64_t a = (int64_t)c.template ld<TA, CI_A + I>(r0, j);
+                if constexpr (S::mode[I] == 3) {
+                    uint64_t v = (uint64_t)a;
+                    if constexpr (MS) v *= (uint64_t)q.sk[I] - (uint64_t)(int64_t)c.template ld<TB, CI_B + I>(r0, j);
+                    v -= (uint64_t)t.sum_off[I];
+                    const uint32_t w[2] = {(uint32_t)v, (uint32_t)(v >> 32)};
+                    add_limbs<3>(p + g[j], t.G, w);
+                } else {
+                    I128 v = i128_from_i64(a);
+                    if constexpr (MS) v = mul_sub(a, q.sk[I], (int64_t)c.template ld<TB, CI_B + I>(r0, j));
+                    const uint32_t w[4] = {(uint32_t)v.lo, (uint32_t)(v.lo >> 32), (uint32_t)v.hi,
+                                           (uint32_t)(v.hi >> 32)};
+                    add_limbs<4>(p + g[j], t.G, w);
+                }
             }
         } else if constexpr (S::fast) {
             uint32_t* lo = (uint32_t*)t.base + (uint64_t)sum_word<S, I>() * t.G;

@@ -59,7 +59,16 @@ template <class S, int I>
 __device__ __forceinline__ void fold_sums(const StageLayout& L, const unsigned char* smem, uint64_t* gacc,
                                           uint32_t G, uint32_t gi, uint64_t cnt) {
     if constexpr (I < S::ns) {
-        if constexpr (S::fast) {
+        if constexpr (S::fast && WideOf<S>::value) {
+            // sum = limbs + count * offset, exact modulo 2^128
+            const uint32_t* w = (const uint32_t*)smem + (uint64_t)L.sum_word[I] * G;
+            unsigned __int128 v = w[gi];
+#pragma unroll
+            for (int i = 1; i < S::mode[I]; ++i) v += (unsigned __int128)w[(uint64_t)i * G + gi] << (32 * i);
+            v += (unsigned __int128)((__int128)L.sum_off[I] * (__int128)cnt);
+            atomic_add_i128(&gacc[(uint64_t)G * (1 + 2 * I) + gi], &gacc[(uint64_t)G * (2 + 2 * I) + gi],
+                            I128{(uint64_t)v, (uint64_t)(v >> 64)});
+        } else if constexpr (S::fast) {
             // sum = carry words * 2^32 + low words + count * offset: exact
             // modulo 2^64 and, by the bounds, inside int64
             const uint32_t* w = (const uint32_t*)smem + (uint64_t)L.sum_word[I] * G;

@@ -233,19 +233,26 @@ struct StageLayout {
     uint32_t table_bytes;              // shared-memory aggregation table in front of the stages
     uint32_t smem_bytes;               // total dynamic shared memory
     uint64_t wait_ns;                  // limit of every mbarrier wait
-    // narrow (32-bit) shared-memory table, used with 64-bit accumulation:
-    // count[G] in word 0, then per sum its low words and, for mode 2, a carry
-    // word block.  Terms are offset by sum_off so they are non-negative.
-    int8_t sum_mode[MAX_SUM];          // 1: low word only, 2: low word + carry word
+    // narrow (32-bit) shared-memory table: count[G] in word 0, then per sum
+    // its blocks of words -- with 64-bit accumulation the low words and, for
+    // mode 2, the carries; wide tables also 3 or 4 limbs of an exact sum.
+    // Terms are offset by sum_off so they are non-negative (mode 4: as they are).
+    int8_t sum_mode[MAX_SUM];          // blocks of G words the sum takes
     uint32_t sum_word[MAX_SUM];        // index (in blocks of G words) of sum s's low words
     int64_t sum_off[MAX_SUM];
 };
 
+#ifndef __CUDACC_RTC__
 // Proven range of one aggregate's per-row term, from column statistics.
 struct TermBounds {
-    int64_t lo;      // minimum term
-    uint64_t span;   // maximum term - minimum term
+    __int128 lo;              // minimum term
+    unsigned __int128 span;   // maximum term - minimum term
 };
+#endif
+// Shared-memory table of a staged aggregation: exact 64-bit words, 32-bit
+// words for sums proved to stay inside int64, 32-bit limbs of exact sums (the
+// run-time compiled dense kernel only).
+enum DenseWords : int32_t { DW_EXACT = 0, DW_FAST = 1, DW_WIDE = 2 };
 
 // --------------------------------------------------------- batched execution
 
@@ -344,16 +351,16 @@ cudaError_t load_plain_kernels();
 
 // Staged shared-memory aggregation.  staged_layout_shared() fills *L for the
 // query (false when the staged kernel cannot run it: misaligned columns,
-// too little shared memory); fast selects 64-bit accumulation.  The launch
+// too little shared memory); DW_FAST selects 64-bit accumulation.  The launch
 // covers the first floor(n / ST_TILE) * ST_TILE rows; the caller runs the
 // remaining rows through launch_agg_shared (64-bit accumulation stays exact
 // there: both keep the same low words, and the high words are ignored).
-// With fast, bounds[s] must give every sum's term range; the layout fails
-// when a 32-bit table cannot hold `rows` rows' worth of sums.
+// Except for DW_EXACT, bounds[s] must give every sum's term range; the layout
+// fails when a 32-bit table cannot hold `rows` rows' worth of sums.
 // geom: the kernel's geometry (the ahead-of-time kernel's is AOT_GEOM);
 // max_stages caps the ring, leaving the shared memory it does not take to
 // the L1 cache.
-bool staged_layout_shared(const QueryDev& q, uint32_t key_bits, bool fast, const TermBounds* bounds,
+bool staged_layout_shared(const QueryDev& q, uint32_t key_bits, DenseWords kind, const TermBounds* bounds,
                           uint64_t rows, int num_sms, const StageGeom& geom, int max_stages, StageLayout* L);
 cudaError_t launch_agg_shared_staged(const QueryDev& q, const StageLayout& L, uint64_t n, uint64_t* gacc,
                                      uint32_t key_bits, bool fast, int num_sms, cudaStream_t st);

@@ -207,7 +207,7 @@ static uint32_t align128(uint64_t x) { return (uint32_t)((x + 127) & ~127ull); }
 
 static int esize_host(int type) { return type == T_I64 ? 8 : (type == T_I32 ? 4 : 1); }
 
-bool staged_layout_shared(const QueryDev& q, uint32_t key_bits, bool fast, const TermBounds* bounds,
+bool staged_layout_shared(const QueryDev& q, uint32_t key_bits, DenseWords kind, const TermBounds* bounds,
                           uint64_t rows, int num_sms, const StageGeom& geom, int max_stages, StageLayout* L) {
     memset(L, 0, sizeof(*L));
     for (int i = 0; i < SL_COUNT; ++i) L->col_of_slot[i] = -1;
@@ -248,7 +248,7 @@ bool staged_layout_shared(const QueryDev& q, uint32_t key_bits, bool fast, const
     }
     L->stage_bytes = off ? off : 128;
     const uint64_t G = 1ull << key_bits;
-    if (fast) {
+    if (kind != DW_EXACT) {
         // rows one CTA can see in this launch bound every 32-bit word: its
         // share of the whole tiles plus, for the run-time compiled kernel, the
         // rows after the last whole tile, which CTA (tiles % grid) evaluates
@@ -259,16 +259,19 @@ bool staged_layout_shared(const QueryDev& q, uint32_t key_bits, bool fast, const
         if (r_cta >= (1ull << 32)) return false;
         uint32_t block = 1;   // block 0: counts
         for (int s = 0; s < q.n_sum; ++s) {
-            const unsigned __int128 rs = (unsigned __int128)r_cta;
-            const uint64_t span = bounds[s].span;
-            if (rs * span <= 0xFFFFFFFFull) {
+            const unsigned __int128 rs = (unsigned __int128)r_cta, span = bounds[s].span;
+            const bool off64 = bounds[s].lo >= INT64_MIN && bounds[s].lo <= INT64_MAX;
+            if (off64 && span <= 0xFFFFFFFFull && rs * span <= 0xFFFFFFFFull) {
                 L->sum_mode[s] = 1;
-            } else if (rs * ((span >> 32) + 1) <= 0xFFFFFFFFull) {
+            } else if (off64 && (span >> 64) == 0 && rs * ((span >> 32) + 1) <= 0xFFFFFFFFull) {
                 L->sum_mode[s] = 2;
+            } else if (kind == DW_WIDE) {
+                // three limbs: fewer than 2^32 rows of terms below 2^64
+                L->sum_mode[s] = off64 && (span >> 64) == 0 ? 3 : 4;
             } else {
                 return false;
             }
-            L->sum_off[s] = bounds[s].lo;
+            L->sum_off[s] = L->sum_mode[s] == 4 ? 0 : (int64_t)bounds[s].lo;
             L->sum_word[s] = block;
             block += (uint32_t)L->sum_mode[s];
         }

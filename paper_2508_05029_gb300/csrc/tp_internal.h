@@ -251,19 +251,20 @@ bool direct_group_range(const tp_plan* p, const tp_table* fact, const tp_table* 
                         uint64_t* span);
 // Column bounds prove every sum of the plan stays inside int64 over the fact table.
 bool sums_fit_int64(const tp_plan* p, const tp_table* fact);
-// Per-row term range of every sum slot (valid when sums_fit_int64 holds).
+// Per-row term range of every sum slot.
 void term_bounds(const tp_plan* p, const tp_table* fact, tpk::TermBounds* out);
 // out[s] = 1 for MUL_SUB sum slots whose two factors fit in int32 by the
 // column statistics.
 void narrow_products(const tp_plan* p, const tp_table* fact, int* out);
 // A plan shape as a struct named `name` of compile-time constants for the
 // run-time compiled kernels; mode[s] is sum s's 32-bit accumulation mode
-// (fast only); lo_only (not fast): 64-bit low-word sums.
+// (fast only); lo_only (not fast): 64-bit low-word sums; wide (fast): sums may
+// leave int64.
 std::string shape_struct(const std::string& name, const tpk::QueryDev& q, const int8_t* mode, bool fast,
-                         bool lo_only, const int* narrow);
+                         bool lo_only, const int* narrow, bool wide = false);
 // The source (shape struct JS and the kernel include) of a dense staged
 // launch's run-time compiled kernel.
-std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, bool fast, const int* narrow);
+std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, tpk::DenseWords kind, const int* narrow);
 // Host-to-device copy of column c of batch b (t's page layout) on `st`: a
 // full-width column lands at full + row_off * size, a narrow one at
 // enc + row_off * size (enc is then widened by widen_batch).  Adds the bytes
