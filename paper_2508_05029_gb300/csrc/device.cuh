@@ -313,7 +313,7 @@ __device__ __forceinline__ bool eval_keys(const QueryDev& q, uint64_t t0, uint64
             for (int i = 0; i < 4; ++i) {
                 if (!pass[i]) continue;
                 const uint64_t at = (uint64_t)payload[i] + m;
-                pass[i] = at < q.jt.mn && __ldg(q.jt.mkeys + at) == (uint64_t)v[i];
+                pass[i] = at < __ldg(q.jt.mn) && __ldg(q.jt.mkeys + at) == (uint64_t)v[i];
                 if (pass[i]) payload[i] = __ldg(q.jt.mpay + at);
             }
         }

@@ -278,46 +278,43 @@ tp_status build_join(ExecState& S, Scratch& sc, int k = 0) {
     }, k);
 }
 
-// Fan-out build of the first join: the admitted rows' (key, payload) pairs
-// sorted by key; the table maps each key to the index of its run's first row.
+// Fan-out build of the first join: the admitted rows grouped by key, the table
+// mapping each key to the index of its run's first row.
 tp_status build_join_many(ExecState& S, Scratch& sc) {
     tp_engine* e = S.e;
     cudaStream_t st = S.lane->compute;
     const uint64_t n_rows = S.dim->rows;
-    void *k0 = nullptr, *v0 = nullptr, *k1 = nullptr, *v1 = nullptr, *hist = nullptr, *hk = nullptr, *hv = nullptr,
-         *ctr = nullptr;
+    void *k0 = nullptr, *v0 = nullptr, *k1 = nullptr, *v1 = nullptr, *pl = nullptr, *ctr = nullptr;
     const uint64_t c = n_rows ? n_rows : 1;
     tp_status s;
     if ((s = sc.alloc(&k0, c * 8)) || (s = sc.alloc(&v0, c * 4)) || (s = sc.alloc(&k1, c * 8)) ||
-        (s = sc.alloc(&v1, c * 4)) || (s = sc.alloc(&hist, tpk::radix_sort_hist_words(c) * 4)) ||
-        (s = sc.alloc(&hk, c * 8)) || (s = sc.alloc(&hv, c * 4)) || (s = sc.alloc(&ctr, 16)))
+        (s = sc.alloc(&v1, c * 4)) || (s = sc.alloc(&pl, c * 8)) || (s = sc.alloc(&ctr, 16)))
         return s;
     TP_TRY_CUDA(cudaMemsetAsync(ctr, 0, 16, st));
-    unsigned long long* cnt = (unsigned long long*)ctr;
+    uint64_t at = 0;   // rows of the batches before
     s = for_each_dim_batch(S, sc, build_proto(S), [&](const tpk::BuildDev& b, uint64_t rows) {
         mark_launch(e);
-        return cuda_check(tpk::launch_many_collect(b, rows, (uint64_t*)k0, (uint32_t*)v0, cnt, e->num_sms, st),
-                          "fan-out build");
+        const uint64_t r0 = at;
+        at += rows;
+        return cuda_check(tpk::launch_many_count(b, rows, (uint64_t*)k0 + r0, (uint32_t*)v0 + r0, (uint64_t*)pl + r0,
+                                                 e->num_sms, st), "fan-out build");
     });
     if (s) return s;
-    TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words, cnt, 8, cudaMemcpyDeviceToHost, st));
-    TP_TRY_CUDA(cudaStreamSynchronize(st));
-    const uint64_t n = S.lane->host_words[0];
-    if (n >= (1ull << 31)) return fail(TP_E_INVALID, "fan-out join: more than 2^31 build rows");
-    uint64_t *kk = (uint64_t*)k0, *tk = (uint64_t*)k1;
-    uint32_t *vv = (uint32_t*)v0, *tv = (uint32_t*)v1;
-    TP_TRY_CUDA(tpk::radix_sort_pairs(&kk, &vv, &tk, &tv, (uint32_t*)hist, n, 64, st));
-    e->launches += 3 * 8;
-    TP_TRY_CUDA(tpk::launch_many_heads(kk, n, (int64_t*)hk, (uint32_t*)hv, cnt + 1, e->num_sms, st));
+    unsigned long long* total = (unsigned long long*)ctr;
+    TP_TRY_CUDA(tpk::launch_many_starts(S.jt, total, e->num_sms, st));
     mark_launch(e);
-    TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words, cnt + 1, 8, cudaMemcpyDeviceToHost, st));
-    TP_TRY_CUDA(cudaStreamSynchronize(st));
-    const uint64_t heads = S.lane->host_words[0];
-    TP_TRY_CUDA(tpk::launch_build_pairs(S.jt, (const int64_t*)hk, (const uint32_t*)hv, heads, S.err, e->num_sms, st));
+    if (n_rows >= (1ull << 31)) {   // only then can too many rows be admitted
+        TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words, total, 8, cudaMemcpyDeviceToHost, st));
+        TP_TRY_CUDA(cudaStreamSynchronize(st));
+        if (S.lane->host_words[0] >= (1ull << 31))
+            return fail(TP_E_INVALID, "fan-out join: more than 2^31 build rows");
+    }
+    TP_TRY_CUDA(tpk::launch_many_place(S.jt, (uint64_t*)k0, (uint32_t*)v0, (uint64_t*)pl, n_rows, (uint64_t*)k1,
+                                       (uint32_t*)v1, e->num_sms, st));
     mark_launch(e);
-    S.jt.mkeys = kk;
-    S.jt.mpay = vv;
-    S.jt.mn = n;
+    S.jt.mkeys = (uint64_t*)k1;
+    S.jt.mpay = (uint32_t*)v1;
+    S.jt.mn = total;
     S.jt.many = 1;
     return TP_OK;
 }
@@ -325,7 +322,7 @@ tp_status build_join_many(ExecState& S, Scratch& sc) {
 // Bytes build_join_many allocates for a dimension of n rows.
 uint64_t many_build_bytes(uint64_t n) {
     const uint64_t c = n ? n : 1;
-    return 3 * align256(c * 8) + 3 * align256(c * 4) + align256(tpk::radix_sort_hist_words(c) * 4) + 256;
+    return 3 * align256(c * 8) + 2 * align256(c * 4) + 256;
 }
 
 // ------------------------------------------------------- fact batch driver

@@ -396,10 +396,11 @@ __device__ __forceinline__ void consume(const QueryDev& q, const Flt& flt, const
         if (!pm) return;
     }
     if constexpr (S::many) {
-        // fan-out: pay[j] is the first row of the key's run in the sorted
-        // build rows; pair the row with each row of the run in turn
+        // fan-out: pay[j] is the first row of the key's run in the
+        // grouped build rows; pair the row with each row of the run in turn
         uint32_t first[ST_RPL];
         int64_t key[ST_RPL];
+        const uint64_t mn = TP_LDT(q.jt.mn);
 #pragma unroll
         for (int j = 0; j < ST_RPL; ++j) {
             first[j] = pay[j];
@@ -411,7 +412,7 @@ __device__ __forceinline__ void consume(const QueryDev& q, const Flt& flt, const
             for (int j = 0; j < ST_RPL; ++j) {
                 if (!((live >> j) & 1u)) continue;
                 const uint64_t at = (uint64_t)first[j] + m;
-                if (at < q.jt.mn && TP_LDT(q.jt.mkeys + at) == (uint64_t)key[j]) pay[j] = TP_LDT(q.jt.mpay + at);
+                if (at < mn && TP_LDT(q.jt.mkeys + at) == (uint64_t)key[j]) pay[j] = TP_LDT(q.jt.mpay + at);
                 else live &= ~(1u << j);
             }
             uint32_t pmm = live, bad = 0;

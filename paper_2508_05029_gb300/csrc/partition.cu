@@ -264,11 +264,68 @@ cudaError_t launch_fact_spill(const QueryDev& q, uint64_t n, uint64_t spill_mask
 }
 
 // ------------------------------------------------------- fan-out build
+//
+// Groups the admitted build rows by key without sorting them: the join table
+// itself counts a key's rows, the counts become run starts, and every row is
+// written at its run's start plus its rank.  Runs come in slot order and rows
+// in no order inside a run, which an inner join's sums do not see.  Three
+// passes over rows or slots, bound by the table's random accesses.  Build and
+// query of 20M fact rows over 1.5M build rows: 1.34 ms per pass when the
+// (key, payload) pairs were sorted by 64 key bits (29 launches, 0.42 ms of
+// kernels and two synchronisations), 0.97 ms grouped this way.
 
-__global__ void k_many_collect(const __grid_constant__ BuildDev b, uint64_t n, uint64_t* __restrict__ keys,
-                               uint32_t* __restrict__ pays, unsigned long long* ctr) {
+// The 32-bit word of table slot s that counts, then holds the start of, its
+// key's run (the slot's payload).
+__device__ __forceinline__ uint32_t* many_word(const JoinTable& jt, uint64_t s) {
+    uint32_t* w = (uint32_t*)jt.slots;
+    return jt.direct ? w + s : (jt.key64 ? w + 4 * s + 2 : w + 2 * s + 1);
+}
+
+// One row's key takes or finds its slot; the row's rank among the key's rows
+// is what the slot's word counted before it.  The words start at all ones
+// (the empty pattern), so a count of c rows reads c - 1.  The key equal to
+// the empty pattern counts in the side cell, from zero.
+__device__ __forceinline__ uint64_t many_insert(const JoinTable& jt, int64_t key, uint32_t* err, uint32_t* rank) {
+    if (jt.direct) {
+        const uint64_t idx = (uint64_t)key - (uint64_t)jt.kmin;
+        if (idx >= jt.range) { atomicOr(err, ERR_INTERNAL); return MANY_NONE; }
+        *rank = atomicAdd(many_word(jt, idx), 1u) + 1u;
+        return idx;
+    }
+    if (jt.key64 ? (uint64_t)key == EMPTY64 : (uint32_t)key == EMPTY32) {
+        jt.side[0] = 1;
+        *rank = atomicAdd(jt.side + 1, 1u);
+        return MANY_SIDE;
+    }
+    uint64_t s = join_hash(jt, key) & jt.mask;
+    for (uint64_t it = 0; it <= jt.mask; ++it) {
+        unsigned long long* p = (unsigned long long*)jt.slots + (jt.key64 ? 2 * s : s);
+        bool mine;
+        if (jt.key64) {
+            const unsigned long long prev = atomicCAS(p, (unsigned long long)EMPTY64, (unsigned long long)key);
+            mine = prev == EMPTY64 || prev == (unsigned long long)key;
+        } else {
+            const unsigned long long prev =
+                atomicCAS(p, (unsigned long long)EMPTY64, ((unsigned long long)EMPTY32 << 32) | (uint32_t)key);
+            mine = (uint32_t)prev == EMPTY32 || (uint32_t)prev == (uint32_t)key;
+        }
+        if (mine) {
+            *rank = atomicAdd(many_word(jt, s), 1u) + 1u;
+            return s;
+        }
+        s = (s + 1) & jt.mask;
+    }
+    atomicOr(err, ERR_INTERNAL);
+    return MANY_NONE;
+}
+
+__global__ void k_many_count(const __grid_constant__ BuildDev b, uint64_t n, uint64_t* __restrict__ keys,
+                             uint32_t* __restrict__ pays, uint64_t* __restrict__ place) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        if (!dim_row_admitted(b, i)) continue;
+        if (!dim_row_admitted(b, i)) {
+            place[i] = MANY_NONE;
+            continue;
+        }
         const int64_t key = ld1(b.key, i);
         if (b.jt.lip != nullptr) lip_insert(b.jt, key);
         uint32_t payload = 0;
@@ -277,37 +334,99 @@ __global__ void k_many_collect(const __grid_constant__ BuildDev b, uint64_t n, u
             if (v < 0 || ((uint64_t)v >> b.dbits[f]) != 0) payload |= PAYLOAD_BAD;
             else payload |= (uint32_t)((uint64_t)v << b.dpos[f]);
         }
-        const unsigned long long at = atomicAdd(ctr, 1ull);
-        keys[at] = (uint64_t)key;
-        pays[at] = payload;
+        uint32_t rank = 0;
+        const uint64_t s = many_insert(b.jt, key, b.err, &rank);
+        keys[i] = (uint64_t)key;
+        pays[i] = payload;
+        place[i] = s == MANY_NONE ? MANY_NONE : (s << MANY_RANK_BITS) | rank;
     }
 }
 
-cudaError_t launch_many_collect(const BuildDev& b, uint64_t n, uint64_t* keys, uint32_t* pays,
-                                unsigned long long* ctr, int num_sms, cudaStream_t st) {
+cudaError_t launch_many_count(const BuildDev& b, uint64_t n, uint64_t* keys, uint32_t* pays, uint64_t* place,
+                              int num_sms, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     uint64_t blocks = (n + 255) / 256;
     if (blocks > (uint64_t)num_sms * 8) blocks = (uint64_t)num_sms * 8;
-    k_many_collect<<<(unsigned)blocks, 256, 0, st>>>(b, n, keys, pays, ctr);
+    k_many_count<<<(unsigned)blocks, 256, 0, st>>>(b, n, keys, pays, place);
     return cudaGetLastError();
 }
 
-__global__ void k_many_heads(const uint64_t* __restrict__ keys, uint64_t n, int64_t* __restrict__ hkeys,
-                             uint32_t* __restrict__ hidx, unsigned long long* ctr) {
+// Turns the counts of the table's slots into run starts; *total ends as the
+// number of rows.  One reservation on *total per tile of MS_TILE slots: one
+// per warp would queue on that word.
+constexpr int MS_THREADS = 256;
+constexpr int MS_ITEMS = 16;
+constexpr int MS_TILE = MS_THREADS * MS_ITEMS;
+
+__global__ void __launch_bounds__(MS_THREADS)
+    k_many_starts(const __grid_constant__ JoinTable jt, uint64_t n_slots, unsigned long long* total) {
+    __shared__ uint32_t warp_sum[MS_THREADS / 32];
+    __shared__ unsigned long long base;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * MS_TILE; t0 < n_slots; t0 += (uint64_t)gridDim.x * MS_TILE) {
+        uint32_t cnt[MS_ITEMS], sum = 0;
+#pragma unroll
+        for (int j = 0; j < MS_ITEMS; ++j) {
+            const uint64_t s = t0 + (uint64_t)j * MS_THREADS + threadIdx.x;
+            cnt[j] = s < n_slots ? *many_word(jt, s) + 1u : 0u;
+            sum += cnt[j];
+        }
+        uint32_t x = sum;
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+        for (int w = 0; w < MS_THREADS / 32; ++w) {
+            if (w < warp) before += warp_sum[w];
+            all += warp_sum[w];
+        }
+        if (threadIdx.x == 0) base = atomicAdd(total, (unsigned long long)all);
+        __syncthreads();
+        uint32_t at = (uint32_t)base + before + x - sum;
+#pragma unroll
+        for (int j = 0; j < MS_ITEMS; ++j) {
+            const uint64_t s = t0 + (uint64_t)j * MS_THREADS + threadIdx.x;
+            if (cnt[j]) *many_word(jt, s) = at;
+            at += cnt[j];
+        }
+        __syncthreads();
+    }
+    // the key equal to the empty pattern
+    if (!jt.direct && blockIdx.x == 0 && threadIdx.x == 0 && jt.side[0] != 0)
+        jt.side[1] = (uint32_t)atomicAdd(total, (unsigned long long)jt.side[1]);
+}
+
+cudaError_t launch_many_starts(const JoinTable& jt, unsigned long long* total, int num_sms, cudaStream_t st) {
+    const uint64_t n_slots = jt.direct ? jt.range : jt.mask + 1;
+    uint64_t blocks = (n_slots + MS_TILE - 1) / MS_TILE;
+    if (blocks > (uint64_t)num_sms * 8) blocks = (uint64_t)num_sms * 8;
+    k_many_starts<<<(unsigned)blocks, MS_THREADS, 0, st>>>(jt, n_slots, total);
+    return cudaGetLastError();
+}
+
+__global__ void k_many_place(const __grid_constant__ JoinTable jt, const uint64_t* __restrict__ keys,
+                             const uint32_t* __restrict__ pays, const uint64_t* __restrict__ place, uint64_t n,
+                             uint64_t* __restrict__ mkeys, uint32_t* __restrict__ mpay) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        if (i > 0 && keys[i] == keys[i - 1]) continue;
-        const unsigned long long at = atomicAdd(ctr, 1ull);
-        hkeys[at] = (int64_t)keys[i];
-        hidx[at] = (uint32_t)i;
+        const uint64_t p = place[i];
+        if (p == MANY_NONE) continue;
+        const uint64_t s = p >> MANY_RANK_BITS;
+        const uint32_t start = s == MANY_SIDE ? jt.side[1] : *many_word(jt, s);
+        const uint64_t at = (uint64_t)start + (p & ((1ull << MANY_RANK_BITS) - 1ull));
+        mkeys[at] = keys[i];
+        mpay[at] = pays[i];
     }
 }
 
-cudaError_t launch_many_heads(const uint64_t* keys, uint64_t n, int64_t* hkeys, uint32_t* hidx,
-                              unsigned long long* ctr, int num_sms, cudaStream_t st) {
+cudaError_t launch_many_place(const JoinTable& jt, const uint64_t* keys, const uint32_t* pays, const uint64_t* place,
+                              uint64_t n, uint64_t* mkeys, uint32_t* mpay, int num_sms, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     uint64_t blocks = (n + 255) / 256;
     if (blocks > (uint64_t)num_sms * 8) blocks = (uint64_t)num_sms * 8;
-    k_many_heads<<<(unsigned)blocks, 256, 0, st>>>(keys, n, hkeys, hidx, ctr);
+    k_many_place<<<(unsigned)blocks, 256, 0, st>>>(jt, keys, pays, place, n, mkeys, mpay);
     return cudaGetLastError();
 }
 
