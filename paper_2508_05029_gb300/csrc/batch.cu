@@ -469,7 +469,7 @@ std::string batch_shape(const tp_plan* p, const tpk::BatchQuery& B, const BatchP
 }
 
 std::string batch_kernel_source(const std::vector<std::string>& shapes) {
-    std::string src;
+    std::string src = geometry_macros(tpk::JIT_DENSE_GEOM);
     for (size_t k = 0; k < shapes.size(); ++k) src += shapes[k];
     src += "#include \"jit_batch.cuh\"\n"
            "__device__ void tpj::dispatch_probe(const tpk::BatchQuery& B, uint64_t r0, uint64_t r1, "

@@ -175,6 +175,58 @@ __device__ __forceinline__ T ld_table(const T* p) {
     else return __ldcg(p);
 }
 
+// Packed hash tables: the word of a key without its payload, in the bucket its
+// lookup starts at (1 << pay_bits more in each bucket after it), that bucket,
+// and the payload of a word.
+__device__ __forceinline__ uint64_t pack_word(const JoinTable& jt, uint64_t h) { return h << jt.cap_bits; }
+__device__ __forceinline__ uint32_t pack_home(const JoinTable& jt, uint64_t h) {
+    return (uint32_t)(h >> (64 - jt.cap_bits));
+}
+__device__ __forceinline__ uint32_t pack_payload(const JoinTable& jt, uint32_t lo) {
+    const uint32_t flag = 1u << (jt.pay_bits - 1);
+    return lo & flag ? PAYLOAD_BAD : lo & (flag - 1u);
+}
+
+// Looks for `word` in one bucket: *lo gets the low half of the match.
+__device__ __forceinline__ bool pack_find(const uint64_t (&w)[4], uint64_t word, uint32_t limit, uint32_t* lo) {
+    const uint32_t hi32 = (uint32_t)(word >> 32), lo32 = (uint32_t)word;
+    bool hit = false;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        if ((uint32_t)(w[m] >> 32) == hi32 && ((uint32_t)w[m] ^ lo32) < limit) {
+            *lo = (uint32_t)w[m];
+            hit = true;
+        }
+    }
+    return hit;
+}
+
+// One key in a packed table: payload | 1 << 32, or 0.  A call of its own: the
+// plain kernels run at their register limit, and four rows' buckets inside
+// them spilled on every path.
+template <bool NC>
+__device__ __noinline__ uint64_t probe1_packed(const uint64_t* slots, uint64_t slot_mask, int cap_bits, int pay_bits,
+                                               int64_t key) {
+    JoinTable jt{};
+    jt.cap_bits = cap_bits;
+    jt.pay_bits = pay_bits;
+    const uint64_t h = fmix64((uint64_t)key);
+    uint32_t at = pack_home(jt, h);
+    uint64_t word = pack_word(jt, h);
+    const uint32_t mask = (uint32_t)(slot_mask >> 2), limit = 1u << pay_bits;
+    for (uint32_t dist = 0; dist <= PACK_MAX_DIST; ++dist) {
+        const ulonglong2* b = (const ulonglong2*)slots + 2 * (uint64_t)at;
+        const ulonglong2 x = ld_table<NC>(b), y = ld_table<NC>(b + 1);
+        const uint64_t w[4] = {x.x, x.y, y.x, y.y};
+        uint32_t lo = 0;
+        if (pack_find(w, word, limit, &lo)) return 1ull << 32 | pack_payload(jt, lo);
+        if (w[3] == EMPTY64) return 0;
+        at = (at + 1) & mask;
+        word += limit;
+    }
+    return 0;
+}
+
 // Looks up four keys at once so their table loads overlap.  pass[i] is
 // cleared for rows whose key is absent.
 template <bool NC = true>
@@ -200,6 +252,17 @@ __device__ __forceinline__ void probe4(const JoinTable& jt, const int64_t key[4]
         for (int i = 0; i < 4; ++i) {
             pass[i] = pass[i] && w[i] != EMPTY32;
             payload[i] = w[i];
+        }
+        return;
+    }
+    if (jt.pay_bits != 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            payload[i] = 0;
+            if (!pass[i]) continue;
+            const uint64_t r = probe1_packed<NC>(jt.slots, jt.mask, jt.cap_bits, jt.pay_bits, key[i]);
+            payload[i] = (uint32_t)r;
+            pass[i] = (r >> 32) != 0;
         }
         return;
     }
@@ -530,6 +593,27 @@ __device__ __forceinline__ void build_insert(const BuildDev& b, uint64_t i) {
         const uint64_t idx = (uint64_t)key - (uint64_t)jt.kmin;
         if (idx >= jt.range) { atomicOr(b.err, ERR_INTERNAL); return; }
         if (atomicCAS((unsigned int*)jt.slots + idx, EMPTY32, v) != EMPTY32) atomicOr(b.err, ERR_DUP);
+        return;
+    }
+    if (jt.pay_bits != 0) {
+        const uint64_t h = fmix64((uint64_t)key);
+        uint32_t at = pack_home(jt, h);
+        uint64_t word = pack_word(jt, h);
+        const uint64_t pay = (payload & PAYLOAD_BAD) ? 1ull << (jt.pay_bits - 1) : (uint64_t)payload;
+        for (uint32_t dist = 0; dist <= PACK_MAX_DIST; ++dist) {
+            unsigned long long* bucket = (unsigned long long*)jt.slots + 4 * (uint64_t)at;
+            for (int m = 0; m < 4; ++m) {
+                const unsigned long long prev =
+                    atomicCAS(bucket + m, (unsigned long long)EMPTY64, (unsigned long long)(word | pay));
+                if (prev == EMPTY64) return;
+                if ((prev ^ word) >> jt.pay_bits == 0) { atomicOr(b.err, ERR_DUP); return; }
+            }
+            // a table far too small for its rows: the first failure ends the others' searches
+            if (dist >= 4 && (*(volatile uint32_t*)b.err & ERR_PACKED)) return;
+            at = (at + 1) & (uint32_t)(jt.mask >> 2);
+            word += 1ull << jt.pay_bits;
+        }
+        atomicOr(b.err, ERR_PACKED);
         return;
     }
     bool special = jt.key64 ? (uint64_t)key == EMPTY64 : (uint32_t)key == EMPTY32;

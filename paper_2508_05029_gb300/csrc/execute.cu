@@ -530,7 +530,12 @@ tp_status sample_dim_selectivity(ExecState& S, int k) {
     return TP_OK;
 }
 
+// Internal status: a packed join table could not hold its rows; the query runs
+// again with unpacked ones.
+constexpr tp_status RETRY_UNPACKED = -1;
+
 tp_status map_err(uint32_t err) {
+    if (err & tpk::ERR_PACKED) return RETRY_UNPACKED;
     if (err & tpk::ERR_DUP) return fail(TP_E_DUP_KEY, "join build side holds a duplicate key");
     if (err & tpk::ERR_RANGE) return fail(TP_E_RANGE, "a group field value does not fit its bit width");
     if (err & tpk::ERR_TIMEOUT) return fail(TP_E_TIMEOUT, "a bounded device wait expired");
@@ -1311,7 +1316,51 @@ tp_status cache_publish(ExecState& S, Scratch& sc, DimCache* c, CacheUse* cu) {
 
 // ------------------------------------------------------------- execution
 
-tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out) {
+// Hashed join table of dimension k: capacity and bytes; pay_bits != 0: packed.
+struct JoinSize {
+    bool key64 = false;
+    uint64_t cap = 0, bytes = 0;
+    int cap_bits = 0, pay_bits = 0;
+};
+
+// 64-bit keys take packed buckets when the payload leaves the distance bits
+// and the expected load is at most PACK_MAX_LOAD, where the longest distance
+// measured over 2^12 .. 2^26 slots was 22 buckets (30 can be recorded; at 0.7
+// it was 38).  A dimension predicate's sampled pass rate (4096 rows, three
+// standard errors up) sizes the table for the admitted rows alone: only packed
+// tables, whose build notices a table that is too small at once.
+constexpr double PACK_MAX_LOAD = 0.6;
+
+JoinSize join_size(const tp_plan* p, int k, bool may_pack) {
+    const tp_table* t = p->dims[k];
+    const double lf = p->load_factor;
+    JoinSize x;
+    x.key64 = t->types[p->joins[k].dim_col] == TP_I64;
+    x.cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)std::ceil(t->rows / lf)));
+    x.bytes = x.cap * (x.key64 ? 16 : 8);
+    if (!x.key64 || !may_pack || p->no_packed) return x;
+    int pay = 1;   // the out-of-range flag
+    for (int g = 0; g < p->d.n_group; ++g)
+        if (p->gdim[g] == k) pay += p->d.group[g].bits;
+    double rows = (double)t->rows;
+    uint64_t cap = x.cap;
+    if (p->dflt[k].col >= 0) {
+        const double sel = std::min(1.0, std::max(0.0, p->dim_sel[k]));
+        rows *= std::min(1.0, sel + 3.0 * std::sqrt(sel * (1.0 - sel) / 4096.0) + 1.0 / 1024.0);
+        cap = std::min(cap, pow2_at_least(std::max<uint64_t>(64, (uint64_t)std::ceil(rows / (lf * 1.25)))));
+    }
+    cap = std::max<uint64_t>(cap, 4ull << std::min(40, pay + (int)tpk::PACK_DIST_BITS));
+    int bits = 0;
+    while ((4ull << bits) < cap) ++bits;
+    if (cap > x.cap || bits > 29 || rows > PACK_MAX_LOAD * (double)cap) return x;
+    x.cap = cap;
+    x.bytes = cap * 8;
+    x.cap_bits = bits;
+    x.pay_bits = pay;
+    return x;
+}
+
+tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out) {
     tp_engine* e = p->eng;
     const tp_plan_desc& d = p->d;
     cudaStream_t st = lane->compute;
@@ -1417,22 +1466,20 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
     // ---- further tables of a star join: always resident, each sized like a
     // first join's unpartitioned table, with its own lookahead filter under
     // the same rule
-    struct XTab {
-        bool direct = false, key64 = false;
-        uint64_t range = 0, cap = 0, bytes = 0, lip_blocks = 0;
+    struct XTab : JoinSize {
+        bool direct = false;
+        uint64_t range = 0, lip_blocks = 0;
     };
     XTab xt[tpk::MAX_XJOIN];
     for (int j = 0; j + 1 < p->n_dims; ++j) {
         tp_table* t = p->dims[1 + j];
         const int kc = p->joins[1 + j].dim_col;
         XTab& x = xt[j];
-        x.key64 = t->types[kc] == TP_I64;
         if (!(e->cfg.flags & TP_FLAG_NO_DIRECT_JOIN) && direct_join_range(t, kc, &x.range)) {
             x.direct = true;
             x.bytes = x.range * 4;
         } else {
-            x.cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)std::ceil(t->rows / lf)));
-            x.bytes = x.cap * (x.key64 ? 16 : 8);
+            (JoinSize&)x = join_size(p, 1 + j, true);
         }
         est += align256(x.bytes);
         if (t->placement == PL_PAGES)   // build staging: key, fields and predicate columns
@@ -1458,8 +1505,13 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
             S.jt.range = range;
             join_bytes = range * 4;
         } else {
-            S.join_cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)std::ceil(S.dim->rows / lf)));
-            join_bytes = S.join_cap * (S.key64 ? 16 : 8);
+            // tables other executions share or partitions split stay unpacked,
+            // and a fan-out's payload is a row index
+            const JoinSize x = join_size(p, 0, !cache && !d.join_many && d.join_partitions <= 1);
+            S.join_cap = x.cap;
+            join_bytes = x.bytes;
+            S.jt.cap_bits = x.cap_bits;
+            S.jt.pay_bits = x.pay_bits;
         }
         full_join_bytes = join_bytes;
         if (lip_possible) {
@@ -1487,6 +1539,7 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
             const int jp = d.join_partitions;
             if (!d.join_many && (jp > 1 || (jp == 0 && join_bytes > avail / 2))) {   // fan-out: never partitioned
                 pj.on = true;
+                S.jt.cap_bits = S.jt.pay_bits = 0;
                 pj.P = jp > 1 ? jp : 64;
                 pj.shift = 64;
                 for (int v = pj.P; v > 1; v >>= 1) --pj.shift;
@@ -1579,6 +1632,8 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
         jt.mask = x.cap ? x.cap - 1 : 0;
         jt.side = (uint32_t*)((uint8_t*)misc + 136 + 8 * j);   // zeroed with misc
         jt.key64 = x.key64 ? 1 : 0;
+        jt.cap_bits = x.cap_bits;
+        jt.pay_bits = x.pay_bits;
         if (x.lip_blocks) {
             void* lip = nullptr;
             if ((s = sc.alloc(&lip, x.lip_blocks * 32))) return s;
@@ -1632,11 +1687,22 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
                     const tpk::DenseWords dw = mode == 2                                 ? tpk::DW_FAST
                                                : (e->cfg.flags & TP_FLAG_EXACT_ONLY) != 0 ? tpk::DW_EXACT
                                                                                           : tpk::DW_WIDE;
-                    if (tpk::staged_layout_shared(q, p->key_bits, dw, bounds, rows, e->num_sms,
-                                                  tpk::JIT_DENSE_GEOM, tpk::JIT_DENSE_STAGES, &LJ) &&
-                        LJ.n_stages == tpk::JIT_DENSE_STAGES && rows >= (uint64_t)LJ.tile) {
+                    bool hashed = q.has_join && !q.jt.direct;
+                    for (int j = 0; j < q.n_xjoin; ++j) hashed = hashed || !q.jtx[j].direct;
+                    auto layout = [&](const tpk::StageGeom& geom, int stages) {
+                        return tpk::staged_layout_shared(q, p->key_bits, dw, bounds, rows, e->num_sms, geom, stages,
+                                                         &LJ) &&
+                               rows >= (uint64_t)LJ.tile;
+                    };
+                    const tpk::StageGeom* geom = nullptr;
+                    if (!hashed && layout(tpk::JIT_DENSE_GEOM, tpk::JIT_DENSE_STAGES) &&
+                        LJ.n_stages == tpk::JIT_DENSE_STAGES)
+                        geom = &tpk::JIT_DENSE_GEOM;
+                    else if (layout(tpk::JIT_HASHED_GEOM, tpk::JIT_HASHED_STAGES))
+                        geom = &tpk::JIT_HASHED_GEOM;
+                    if (geom) {
                         std::string why;
-                        jk = jit_kernel(e, dense_shape(q, LJ, dw, narrow), "tpj_dense", &why);
+                        jk = jit_kernel(e, dense_shape(q, LJ, *geom, dw, narrow), "tpj_dense", &why);
                         if (jk) {
                             L = LJ;   // the ahead-of-time kernel keeps its own layout
                             e->jit_launches++;
@@ -1977,6 +2043,16 @@ tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** ou
     return TP_OK;
 }
 
+tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out) {
+    tp_status s = execute_once(p, lane, cache, out);
+    if (s == RETRY_UNPACKED) {   // Section 3.3.2: a task retried with a better estimate
+        p->no_packed = true;
+        p->eng->retries++;
+        s = execute_once(p, lane, cache, out);
+    }
+    return s;
+}
+
 }  // namespace
 
 namespace tp {
@@ -2122,10 +2198,11 @@ std::string shape_struct(const std::string& name, const tpk::QueryDev& q, const 
         mode[s] = fast ? mode_in[s] : 0;
         nar[s] = fast && mode[s] == 2 && q.skind[s] == tpk::S_MUL_SUB ? narrow[s] : 0;
     }
-    const int join = !q.has_join ? 0 : (q.jt.direct ? 1 : (q.jt.key64 ? 3 : 2));
+    auto kind = [](const tpk::JoinTable& t) { return t.direct ? 1 : (t.pay_bits ? 4 : (t.key64 ? 3 : 2)); };
+    const int join = !q.has_join ? 0 : kind(q.jt);
     int xjoin[tpk::MAX_XJOIN] = {}, xktype[tpk::MAX_XJOIN] = {}, xlip[tpk::MAX_XJOIN] = {}, gdim[tpk::MAX_GROUP] = {};
     for (int j = 0; j < q.n_xjoin; ++j) {
-        xjoin[j] = q.jtx[j].direct ? 1 : (q.jtx[j].key64 ? 3 : 2);
+        xjoin[j] = kind(q.jtx[j]);
         xktype[j] = q.fkx[j].type;
         xlip[j] = q.jtx[j].lip != nullptr ? 1 : 0;
     }
@@ -2152,8 +2229,14 @@ std::string shape_struct(const std::string& name, const tpk::QueryDev& q, const 
 }
 
 // The source of a dense staged launch's run-time compiled kernel.
-std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, tpk::DenseWords kind, const int* narrow) {
-    return shape_struct("JS", q, L.sum_mode, kind != tpk::DW_EXACT, false, narrow, kind == tpk::DW_WIDE) +
+std::string geometry_macros(const tpk::StageGeom& geom) {
+    return "#define TP_ST_CONSUMERS " + std::to_string(geom.consumers) + "\n#define TP_ST_RPL " +
+           std::to_string(geom.rpl) + "\n#define TP_ST_CTAS " + std::to_string(geom.ctas) + "\n";
+}
+
+std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, const tpk::StageGeom& geom,
+                        tpk::DenseWords kind, const int* narrow) {
+    return geometry_macros(geom) + shape_struct("JS", q, L.sum_mode, kind != tpk::DW_EXACT, false, narrow, kind == tpk::DW_WIDE) +
            "#include \"jit_dense.cuh\"\n";
 }
 

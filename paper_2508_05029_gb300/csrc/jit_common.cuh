@@ -10,7 +10,7 @@
 //
 // A shape S provides:
 //   filter, ftype            filter present; its column type (T_*)
-//   join, ktype              J_NONE / J_DIRECT / J_HASH32 / J_HASH64; fk type
+//   join, ktype              J_NONE / J_DIRECT / J_HASH32 / J_HASH64 / J_PACKED64; fk type
 //   part                     partition filter on the join (hybrid join)
 //   lip                      lookahead (Bloom) filter tested before the probe
 //   nx, xjoin[], xktype[], xlip[]   further joins of a star query: kind, key
@@ -45,7 +45,7 @@
 namespace tpj {
 using namespace tpk;
 
-enum : int { J_NONE = 0, J_DIRECT = 1, J_HASH32 = 2, J_HASH64 = 3 };
+enum : int { J_NONE = 0, J_DIRECT = 1, J_HASH32 = 2, J_HASH64 = 3, J_PACKED64 = 4 };
 
 template <int T> struct ColT;
 template <> struct ColT<T_I32> { using type = int32_t; using utype = uint32_t; };
@@ -312,6 +312,8 @@ __device__ __forceinline__ void further_joins(const QueryDev& q, const C& c, uin
                 if (pay[j] == EMPTY32) pm &= ~(1u << j);
         } else if constexpr (S::xjoin[J] == J_HASH32) {
             probe_rows_k32(jt, key, pm, pay, q.err);
+        } else if constexpr (S::xjoin[J] == J_PACKED64) {
+            probe_rows_packed(jt, key, pm, pay);
         } else {
             probe_rows_k64(jt, key, pm, pay, q.err);
         }
@@ -369,7 +371,7 @@ __device__ __forceinline__ void consume(const QueryDev& q, const Flt& flt, const
 #pragma unroll
         for (int j = 0; j < ST_RPL; ++j)
             if (pay[j] == EMPTY32) pm &= ~(1u << j);
-    } else if constexpr (S::join == J_HASH32 || S::join == J_HASH64) {
+    } else if constexpr (S::join != J_NONE) {
         int64_t key[ST_RPL];
 #pragma unroll
         for (int j = 0; j < ST_RPL; ++j) key[j] = (int64_t)c.template ld<S::ktype, CI_K>(r0, j);
@@ -378,7 +380,8 @@ __device__ __forceinline__ void consume(const QueryDev& q, const Flt& flt, const
             for (int j = 0; j < ST_RPL; ++j)
                 if (!part_resident(q.jt, key[j])) pm &= ~(1u << j);
         }
-        if constexpr (S::join == J_HASH32) probe_rows_k32(q.jt, key, pm, pay, q.err);
+        if constexpr (S::join == J_PACKED64) probe_rows_packed(q.jt, key, pm, pay);
+        else if constexpr (S::join == J_HASH32) probe_rows_k32(q.jt, key, pm, pay, q.err);
         else probe_rows_k64(q.jt, key, pm, pay, q.err);
     }
     if constexpr (S::join != J_NONE) {

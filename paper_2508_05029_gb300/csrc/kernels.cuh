@@ -37,6 +37,7 @@ enum : uint32_t {
     ERR_OVERFLOW = 4u,   // aggregation table full: execution must be retried larger
     ERR_INTERNAL = 8u,   // probe ran past the table size (cannot happen below full load)
     ERR_TIMEOUT = 16u,   // a bounded device wait expired
+    ERR_PACKED = 32u,    // a packed join table could not place a key: rerun with unpacked tables
 };
 
 constexpr uint64_t EMPTY64 = ~0ull;
@@ -58,6 +59,17 @@ struct DevCol {
 //   all ones.  64-bit keys: two words per slot {key, payload}, EMPTY key = all
 //   ones.  A key equal to the EMPTY pattern lives in side[]: side[0] = 1 when
 //   present, side[1] = its payload.
+//   Packed hash (pay_bits != 0, 64-bit keys): buckets of four 64-bit words, one
+//   aligned 32-byte sector each.  fmix64 is a bijection, so a key is its hash,
+//   and the bucket a lookup starts at is the hash's top cap_bits: a word keeps
+//   the other hash bits, how many buckets it lies past that one, the payload,
+//     hash bits [64 - cap_bits) << cap_bits | distance << pay_bits | payload,
+//   the payload's highest bit marking an out-of-range field.  Keys compare
+//   exactly in half the bytes of {key, payload} slots, four to a sector.  A
+//   bucket fills from its first word and a key goes to the next bucket only
+//   when one is full, at most PACK_MAX_DIST buckets on (ERR_PACKED when those
+//   are full): a lookup ends at a bucket whose last word is empty.  EMPTY = all
+//   ones, which no entry equals (the largest distance is not used).
 //   Direct (dense keys: the key range is at most twice the row count): one
 //   32-bit payload word per key in [kmin, kmin + range), at slot key - kmin;
 //   EMPTY32 = absent (an out-of-range payload is stored as exactly
@@ -75,13 +87,13 @@ struct JoinTable {
     // zero-initialised default) means no partition filter
     uint64_t part_mask;
     int32_t part_shift;
-    int32_t pad2;
+    int32_t cap_bits;       // packed hash: log2(buckets)
     // lookahead filter (lip != nullptr): a blocked Bloom filter of the
     // admitted build keys, 8 words per block; a key's block is
     // fmix64(key) >> lip_shift
     uint32_t* lip;
     int32_t lip_shift;
-    int32_t pad3;
+    int32_t pay_bits;       // packed hash: payload bits and the out-of-range flag; 0 otherwise
     // fan-out (many != 0, repeated build keys): the table maps a key to the
     // index of its first row in mkeys/mpay, the *mn admitted build rows
     // grouped by key; a fact row pairs with rows first, first + 1, ... while
@@ -92,6 +104,9 @@ struct JoinTable {
     int32_t many;
     int32_t pad4;
 };
+
+constexpr uint32_t PACK_DIST_BITS = 5;                            // at least this many distance bits
+constexpr uint32_t PACK_MAX_DIST = (1u << PACK_DIST_BITS) - 2;
 
 // The query as the per-batch kernels see it.  Column pointers address the
 // current batch (row 0 = first row of the batch).
@@ -214,6 +229,18 @@ constexpr StageGeom AOT_GEOM{ST_CONSUMERS, ST_RPL, ST_CTAS};
 // copies).
 constexpr StageGeom JIT_DENSE_GEOM{24, 2, 1};
 constexpr int JIT_DENSE_STAGES = 3;
+// The same kernel when a join is hashed, or when three of those stages do not
+// fit: one row per lane and as many warps as a CTA takes, at most four
+// stages.  A hashed lookup is a chain of dependent sector loads, each holding
+// an L1 line while it is in flight: fewer rows per lane shorten a tile's
+// longest chain and smaller stages leave L1 for the lines.  60M rows, one
+// hashed join / a direct and a hashed one with its lookahead filter, query
+// time: {24, 2, 1} x 3 stages 636 / 1633 us, x 2 stages 701 / 1322; {31, 2, 1}
+// x 2 672 / 1344; {24, 1, 2} x 3 601 / does not fit; {31, 1, 1} x 3 621 / 1304,
+// x 4 588 / 1297, x 6 635 / does not fit.  The direct join keeps its own: 405
+// us against 420 and more with other splits.
+constexpr StageGeom JIT_HASHED_GEOM{31, 1, 1};
+constexpr int JIT_HASHED_STAGES = 4;
 // column slots of a QueryDev: filter, fk, 4 group columns, 8 + 8 sum columns
 enum : int { SL_FILTER = 0, SL_FK = 1, SL_GROUP = 2, SL_SA = 6, SL_SB = 14, SL_FKX = 22, SL_COUNT = 25 };
 

@@ -174,6 +174,7 @@ struct tp_plan {
     tp_filter dflt[4] = {};
     double dim_sel[4] = {-1.0, -1.0, -1.0, -1.0};   // sampled predicate pass rates
     int gdim[4] = {-1, -1, -1, -1};                 // dimension of group field g, -1: fact
+    bool no_packed = false;      // a packed join table could not place a key: unpacked ones from then on
 };
 
 struct tp_result {
@@ -262,9 +263,12 @@ void narrow_products(const tp_plan* p, const tp_table* fact, int* out);
 // leave int64.
 std::string shape_struct(const std::string& name, const tpk::QueryDev& q, const int8_t* mode, bool fast,
                          bool lo_only, const int* narrow, bool wide = false);
-// The source (shape struct JS and the kernel include) of a dense staged
-// launch's run-time compiled kernel.
-std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, tpk::DenseWords kind, const int* narrow);
+// The source (geometry, shape struct JS and the kernel include) of a dense
+// staged launch's run-time compiled kernel; the layout was sized for geom.
+std::string dense_shape(const tpk::QueryDev& q, const tpk::StageLayout& L, const tpk::StageGeom& geom,
+                        tpk::DenseWords kind, const int* narrow);
+// The macros that give a run-time compiled kernel its geometry.
+std::string geometry_macros(const tpk::StageGeom& geom);
 // Host-to-device copy of column c of batch b (t's page layout) on `st`: a
 // full-width column lands at full + row_off * size, a narrow one at
 // enc + row_off * size (enc is then widened by widen_batch).  Adds the bytes
