@@ -375,9 +375,11 @@ __device__ __forceinline__ bool eval_keys(const QueryDev& q, uint64_t t0, uint64
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 if (!pass[i]) continue;
-                const uint64_t at = (uint64_t)payload[i] + m;
-                pass[i] = at < __ldg(q.jt.mn) && __ldg(q.jt.mkeys + at) == (uint64_t)v[i];
-                if (pass[i]) payload[i] = __ldg(q.jt.mpay + at);
+                const uint32_t first = payload[i];
+                const uint2 r = __ldg(q.jt.mrow + first);
+                pass[i] = m <= r.y;
+                payload[i] = r.x;
+                if (pass[i] && m != 0) payload[i] = __ldg(&q.jt.mrow[(uint64_t)first + m].x);
             }
         }
 #pragma unroll

@@ -284,11 +284,11 @@ tp_status build_join_many(ExecState& S, Scratch& sc) {
     tp_engine* e = S.e;
     cudaStream_t st = S.lane->compute;
     const uint64_t n_rows = S.dim->rows;
-    void *k0 = nullptr, *v0 = nullptr, *k1 = nullptr, *v1 = nullptr, *pl = nullptr, *ctr = nullptr;
+    void *pays = nullptr, *place = nullptr, *rows_out = nullptr, *ctr = nullptr;
     const uint64_t c = n_rows ? n_rows : 1;
     tp_status s;
-    if ((s = sc.alloc(&k0, c * 8)) || (s = sc.alloc(&v0, c * 4)) || (s = sc.alloc(&k1, c * 8)) ||
-        (s = sc.alloc(&v1, c * 4)) || (s = sc.alloc(&pl, c * 8)) || (s = sc.alloc(&ctr, 16)))
+    if ((s = sc.alloc(&pays, c * 4)) || (s = sc.alloc(&place, c * 8)) || (s = sc.alloc(&rows_out, c * 8)) ||
+        (s = sc.alloc(&ctr, 16)))
         return s;
     TP_TRY_CUDA(cudaMemsetAsync(ctr, 0, 16, st));
     uint64_t at = 0;   // rows of the batches before
@@ -296,12 +296,12 @@ tp_status build_join_many(ExecState& S, Scratch& sc) {
         mark_launch(e);
         const uint64_t r0 = at;
         at += rows;
-        return cuda_check(tpk::launch_many_count(b, rows, (uint64_t*)k0 + r0, (uint32_t*)v0 + r0, (uint64_t*)pl + r0,
-                                                 e->num_sms, st), "fan-out build");
+        return cuda_check(tpk::launch_many_count(b, rows, (uint32_t*)pays + r0, (uint64_t*)place + r0, e->num_sms, st),
+                          "fan-out build");
     });
     if (s) return s;
     unsigned long long* total = (unsigned long long*)ctr;
-    TP_TRY_CUDA(tpk::launch_many_starts(S.jt, total, e->num_sms, st));
+    TP_TRY_CUDA(tpk::launch_many_starts(S.jt, (uint2*)rows_out, total, e->num_sms, st));
     mark_launch(e);
     if (n_rows >= (1ull << 31)) {   // only then can too many rows be admitted
         TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words, total, 8, cudaMemcpyDeviceToHost, st));
@@ -309,12 +309,10 @@ tp_status build_join_many(ExecState& S, Scratch& sc) {
         if (S.lane->host_words[0] >= (1ull << 31))
             return fail(TP_E_INVALID, "fan-out join: more than 2^31 build rows");
     }
-    TP_TRY_CUDA(tpk::launch_many_place(S.jt, (uint64_t*)k0, (uint32_t*)v0, (uint64_t*)pl, n_rows, (uint64_t*)k1,
-                                       (uint32_t*)v1, e->num_sms, st));
+    TP_TRY_CUDA(tpk::launch_many_place(S.jt, (uint32_t*)pays, (uint64_t*)place, n_rows, (uint2*)rows_out, e->num_sms,
+                                       st));
     mark_launch(e);
-    S.jt.mkeys = (uint64_t*)k1;
-    S.jt.mpay = (uint32_t*)v1;
-    S.jt.mn = total;
+    S.jt.mrow = (uint2*)rows_out;
     S.jt.many = 1;
     return TP_OK;
 }
@@ -322,7 +320,7 @@ tp_status build_join_many(ExecState& S, Scratch& sc) {
 // Bytes build_join_many allocates for a dimension of n rows.
 uint64_t many_build_bytes(uint64_t n) {
     const uint64_t c = n ? n : 1;
-    return 3 * align256(c * 8) + 2 * align256(c * 4) + 256;
+    return 2 * align256(c * 8) + align256(c * 4) + 256;
 }
 
 // ------------------------------------------------------- fact batch driver

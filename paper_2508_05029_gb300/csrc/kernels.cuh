@@ -95,12 +95,10 @@ struct JoinTable {
     int32_t lip_shift;
     int32_t pay_bits;       // packed hash: payload bits and the out-of-range flag; 0 otherwise
     // fan-out (many != 0, repeated build keys): the table maps a key to the
-    // index of its first row in mkeys/mpay, the *mn admitted build rows
-    // grouped by key; a fact row pairs with rows first, first + 1, ... while
-    // mkeys holds its key
-    const uint64_t* mkeys;
-    const uint32_t* mpay;
-    const unsigned long long* mn;
+    // index of its first row in mrow, the admitted build rows grouped by key:
+    // x = the row's payload; y, in the first row of a key's run, = how many
+    // rows of the run follow it
+    const uint2* mrow;
     int32_t many;
     int32_t pad4;
 };
@@ -429,18 +427,19 @@ cudaError_t launch_part_hist(const BuildDev& b, uint64_t n, int shift, unsigned 
                              cudaStream_t st);
 // Fan-out build, fewer than 2^31 admitted rows: launch_many_count inserts the
 // admitted rows' keys into b.jt (its words all ones) and the lookahead filter
-// and writes every row's key, payload and place (table slot << MANY_RANK_BITS
-// | rank among the key's rows; MANY_NONE: not admitted), launch_many_starts
-// makes the slots' payloads the starts of their keys' runs (*total: rows), and
-// launch_many_place writes the rows into the runs.
+// and writes every row's payload and place (table slot << MANY_RANK_BITS |
+// rank among the key's rows; MANY_NONE: not admitted), launch_many_starts
+// makes the slots' payloads the starts of their keys' runs and writes the runs'
+// lengths (*total: rows), and launch_many_place writes the rows into the runs.
 constexpr int MANY_RANK_BITS = 31;
 constexpr uint64_t MANY_NONE = ~0ull;
 constexpr uint64_t MANY_SIDE = (1ull << (64 - MANY_RANK_BITS)) - 2;   // the side cell's rows
-cudaError_t launch_many_count(const BuildDev& b, uint64_t n, uint64_t* keys, uint32_t* pays, uint64_t* place,
-                              int num_sms, cudaStream_t st);
-cudaError_t launch_many_starts(const JoinTable& jt, unsigned long long* total, int num_sms, cudaStream_t st);
-cudaError_t launch_many_place(const JoinTable& jt, const uint64_t* keys, const uint32_t* pays, const uint64_t* place,
-                              uint64_t n, uint64_t* mkeys, uint32_t* mpay, int num_sms, cudaStream_t st);
+cudaError_t launch_many_count(const BuildDev& b, uint64_t n, uint32_t* pays, uint64_t* place, int num_sms,
+                              cudaStream_t st);
+cudaError_t launch_many_starts(const JoinTable& jt, uint2* rows, unsigned long long* total, int num_sms,
+                               cudaStream_t st);
+cudaError_t launch_many_place(const JoinTable& jt, const uint32_t* pays, const uint64_t* place, uint64_t n,
+                              uint2* rows, int num_sms, cudaStream_t st);
 cudaError_t launch_part_hist_fact(const QueryDev& q, uint64_t n, int shift, uint64_t spill_mask,
                                   unsigned long long* counts, int num_sms, cudaStream_t st);
 // Build side: rows of resident partitions (bit set in b.jt.part_mask) are

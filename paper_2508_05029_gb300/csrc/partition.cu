@@ -319,8 +319,8 @@ __device__ __forceinline__ uint64_t many_insert(const JoinTable& jt, int64_t key
     return MANY_NONE;
 }
 
-__global__ void k_many_count(const __grid_constant__ BuildDev b, uint64_t n, uint64_t* __restrict__ keys,
-                             uint32_t* __restrict__ pays, uint64_t* __restrict__ place) {
+__global__ void k_many_count(const __grid_constant__ BuildDev b, uint64_t n, uint32_t* __restrict__ pays,
+                             uint64_t* __restrict__ place) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         if (!dim_row_admitted(b, i)) {
             place[i] = MANY_NONE;
@@ -336,18 +336,17 @@ __global__ void k_many_count(const __grid_constant__ BuildDev b, uint64_t n, uin
         }
         uint32_t rank = 0;
         const uint64_t s = many_insert(b.jt, key, b.err, &rank);
-        keys[i] = (uint64_t)key;
         pays[i] = payload;
         place[i] = s == MANY_NONE ? MANY_NONE : (s << MANY_RANK_BITS) | rank;
     }
 }
 
-cudaError_t launch_many_count(const BuildDev& b, uint64_t n, uint64_t* keys, uint32_t* pays, uint64_t* place,
-                              int num_sms, cudaStream_t st) {
+cudaError_t launch_many_count(const BuildDev& b, uint64_t n, uint32_t* pays, uint64_t* place, int num_sms,
+                              cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     uint64_t blocks = (n + 255) / 256;
     if (blocks > (uint64_t)num_sms * 8) blocks = (uint64_t)num_sms * 8;
-    k_many_count<<<(unsigned)blocks, 256, 0, st>>>(b, n, keys, pays, place);
+    k_many_count<<<(unsigned)blocks, 256, 0, st>>>(b, n, pays, place);
     return cudaGetLastError();
 }
 
@@ -359,7 +358,8 @@ constexpr int MS_ITEMS = 16;
 constexpr int MS_TILE = MS_THREADS * MS_ITEMS;
 
 __global__ void __launch_bounds__(MS_THREADS)
-    k_many_starts(const __grid_constant__ JoinTable jt, uint64_t n_slots, unsigned long long* total) {
+    k_many_starts(const __grid_constant__ JoinTable jt, uint64_t n_slots, uint2* __restrict__ rows,
+                  unsigned long long* total) {
     __shared__ uint32_t warp_sum[MS_THREADS / 32];
     __shared__ unsigned long long base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -389,44 +389,48 @@ __global__ void __launch_bounds__(MS_THREADS)
 #pragma unroll
         for (int j = 0; j < MS_ITEMS; ++j) {
             const uint64_t s = t0 + (uint64_t)j * MS_THREADS + threadIdx.x;
-            if (cnt[j]) *many_word(jt, s) = at;
+            if (cnt[j]) {
+                *many_word(jt, s) = at;
+                rows[at].y = cnt[j] - 1u;
+            }
             at += cnt[j];
         }
         __syncthreads();
     }
     // the key equal to the empty pattern
-    if (!jt.direct && blockIdx.x == 0 && threadIdx.x == 0 && jt.side[0] != 0)
-        jt.side[1] = (uint32_t)atomicAdd(total, (unsigned long long)jt.side[1]);
+    if (!jt.direct && blockIdx.x == 0 && threadIdx.x == 0 && jt.side[0] != 0) {
+        const uint32_t n = jt.side[1], at = (uint32_t)atomicAdd(total, (unsigned long long)n);
+        rows[at].y = n - 1u;
+        jt.side[1] = at;
+    }
 }
 
-cudaError_t launch_many_starts(const JoinTable& jt, unsigned long long* total, int num_sms, cudaStream_t st) {
+cudaError_t launch_many_starts(const JoinTable& jt, uint2* rows, unsigned long long* total, int num_sms,
+                               cudaStream_t st) {
     const uint64_t n_slots = jt.direct ? jt.range : jt.mask + 1;
     uint64_t blocks = (n_slots + MS_TILE - 1) / MS_TILE;
     if (blocks > (uint64_t)num_sms * 8) blocks = (uint64_t)num_sms * 8;
-    k_many_starts<<<(unsigned)blocks, MS_THREADS, 0, st>>>(jt, n_slots, total);
+    k_many_starts<<<(unsigned)blocks, MS_THREADS, 0, st>>>(jt, n_slots, rows, total);
     return cudaGetLastError();
 }
 
-__global__ void k_many_place(const __grid_constant__ JoinTable jt, const uint64_t* __restrict__ keys,
-                             const uint32_t* __restrict__ pays, const uint64_t* __restrict__ place, uint64_t n,
-                             uint64_t* __restrict__ mkeys, uint32_t* __restrict__ mpay) {
+__global__ void k_many_place(const __grid_constant__ JoinTable jt, const uint32_t* __restrict__ pays,
+                             const uint64_t* __restrict__ place, uint64_t n, uint2* __restrict__ rows) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t p = place[i];
         if (p == MANY_NONE) continue;
         const uint64_t s = p >> MANY_RANK_BITS;
         const uint32_t start = s == MANY_SIDE ? jt.side[1] : *many_word(jt, s);
-        const uint64_t at = (uint64_t)start + (p & ((1ull << MANY_RANK_BITS) - 1ull));
-        mkeys[at] = keys[i];
-        mpay[at] = pays[i];
+        rows[(uint64_t)start + (p & ((1ull << MANY_RANK_BITS) - 1ull))].x = pays[i];
     }
 }
 
-cudaError_t launch_many_place(const JoinTable& jt, const uint64_t* keys, const uint32_t* pays, const uint64_t* place,
-                              uint64_t n, uint64_t* mkeys, uint32_t* mpay, int num_sms, cudaStream_t st) {
+cudaError_t launch_many_place(const JoinTable& jt, const uint32_t* pays, const uint64_t* place, uint64_t n,
+                              uint2* rows, int num_sms, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     uint64_t blocks = (n + 255) / 256;
     if (blocks > (uint64_t)num_sms * 8) blocks = (uint64_t)num_sms * 8;
-    k_many_place<<<(unsigned)blocks, 256, 0, st>>>(jt, keys, pays, place, n, mkeys, mpay);
+    k_many_place<<<(unsigned)blocks, 256, 0, st>>>(jt, pays, place, n, rows);
     return cudaGetLastError();
 }
 
