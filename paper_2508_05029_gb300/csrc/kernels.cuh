@@ -38,6 +38,7 @@ enum : uint32_t {
     ERR_INTERNAL = 8u,   // probe ran past the table size (cannot happen below full load)
     ERR_TIMEOUT = 16u,   // a bounded device wait expired
     ERR_PACKED = 32u,    // a packed join table could not place a key: rerun with unpacked tables
+    ERR_RECORDS = 64u,   // a record partition or its table is full: aggregate through the global table
 };
 
 constexpr uint64_t EMPTY64 = ~0ull;
@@ -176,6 +177,36 @@ struct AggTable {
     int32_t pad2;
 };
 
+// Records of a many-group aggregation, in n_part key ranges of 2^shift keys
+// from kmin (records.cu).  A partition keeps its records in REC_WAYS lists, a
+// warp appending to one of them, so that fewer warps queue on a list's cursor:
+// list l = p * REC_WAYS + way holds cursor[l * REC_CURSOR_STRIDE] records (more
+// than cap: ERR_RECORDS).  r0 = {key inside the partition, rows,
+// low and high word of sum 0}, sum[s] = sum s > 0, of the rows' terms modulo
+// 2^64 (column bounds proved the sums stay inside int64).  Record i of list l
+// lies at rec_at(): chunks of REC_CHUNK records, chunk k of every list before
+// chunk k + 1 of any.  Partitions that fill evenly write
+// into one narrow band at a time; with a region per partition every record
+// went to another page of a buffer of a GB or more.
+constexpr uint32_t REC_CURSOR_STRIDE = 16;   // words between cursors: one sector pair each
+constexpr uint32_t REC_MAX_PART = 4096;
+constexpr int REC_HASH_BITS = 12;
+constexpr uint32_t REC_HASH = 1u << REC_HASH_BITS;   // slots of a hashed partition's table
+constexpr int REC_MAX_SUM = 4;
+constexpr uint32_t REC_CHUNK = 128;
+constexpr uint32_t REC_WAYS = 4;
+constexpr int HLL_BITS = 12;
+constexpr uint32_t HLL_REGS = 1u << HLL_BITS;
+struct RecDev {
+    uint4* r0;
+    uint64_t* sum[REC_MAX_SUM];
+    uint32_t* cursor;
+    uint64_t kmin, span;    // keys lie in [kmin, kmin + span)
+    uint32_t n_part, cap;   // cap: records of a list
+    int32_t shift;
+    int32_t pad;
+};
+
 // Output arrays of one result (device memory).
 struct OutDev {
     uint64_t* keys;
@@ -239,6 +270,8 @@ constexpr int JIT_DENSE_STAGES = 3;
 // us against 420 and more with other splits.
 constexpr StageGeom JIT_HASHED_GEOM{31, 1, 1};
 constexpr int JIT_HASHED_STAGES = 4;
+// The run-time compiled record scan: four rows per thread (records.cuh).
+constexpr StageGeom JIT_RECORDS_GEOM{8, 4, 1};
 // column slots of a QueryDev: filter, fk, 4 group columns, 8 + 8 sum columns
 enum : int { SL_FILTER = 0, SL_FK = 1, SL_GROUP = 2, SL_SA = 6, SL_SB = 14, SL_FKX = 22, SL_COUNT = 25 };
 
@@ -416,6 +449,32 @@ cudaError_t launch_select(const QueryDev& q, uint64_t n, uint32_t* sel, unsigned
                           cudaStream_t st);
 cudaError_t launch_agg_selected(const QueryDev& q, const uint32_t* sel, const unsigned long long* count,
                                 uint64_t max_rows, const AggTable& t, bool fast, int num_sms, cudaStream_t st);
+
+// ------------------------------------------------- partitioned aggregation
+//
+// Group fields all in the fact table, no further joins, no fan-out, n_sum <=
+// REC_MAX_SUM, fewer than 2^32 rows, 16-byte aligned columns.
+cudaError_t launch_rec_scan(const QueryDev& q, uint64_t n, const RecDev& rec, int num_sms, cudaStream_t st);
+// The same launch of a run-time compiled scan (tpj_records).
+cudaError_t launch_rec_scan_jit(const void* kernel, const QueryDev& q, uint64_t n, const RecDev& rec, int num_sms,
+                                cudaStream_t st);
+// The *count rows of a selection vector (launch_select), at most max_rows.
+cudaError_t launch_rec_selected(const QueryDev& q, const uint32_t* sel, const unsigned long long* count,
+                                uint64_t max_rows, const RecDev& rec, int num_sms, cudaStream_t st);
+// Groups of every partition, in key order, over its records; groups[p] = their
+// number.  hashed: partitions of more keys than shared memory addresses
+// (shift <= 31), otherwise rec_direct_smem(shift, n_sum) must fit.
+cudaError_t launch_rec_aggregate(const RecDev& rec, int n_sum, bool hashed, uint32_t* groups, uint32_t* err,
+                                 int num_sms, cudaStream_t st);
+uint32_t rec_direct_smem(int shift, int n_sum);
+cudaError_t launch_rec_emit(const RecDev& rec, int n_sum, const uint32_t* groups, const unsigned long long* offsets,
+                            const OutDev& o, int num_sms, cudaStream_t st);
+// Of `samples` evenly spaced rows: out[0] = those passing the filter, out[1] =
+// the most of them in one partition.
+cudaError_t launch_rec_sample(const QueryDev& q, uint64_t n, uint32_t samples, const RecDev& rec,
+                              unsigned long long* out, cudaStream_t st);
+// HyperLogLog registers (HLL_REGS words, zeroed) of the rows' group keys.
+cudaError_t launch_rec_distinct(const QueryDev& q, uint64_t n, uint32_t* regs, int num_sms, cudaStream_t st);
 
 // ------------------------------------------------------- partitioned join
 //

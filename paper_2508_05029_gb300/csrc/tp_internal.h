@@ -174,6 +174,9 @@ struct tp_plan {
     tp_filter dflt[4] = {};
     double dim_sel[4] = {-1.0, -1.0, -1.0, -1.0};   // sampled predicate pass rates
     int gdim[4] = {-1, -1, -1, -1};                 // dimension of group field g, -1: fact
+    uint64_t distinct_groups = 0;   // estimated distinct group keys of the fact table, 0 until measured
+    double rec_skew = -1.0;         // sampled: fullest key partition over the mean, < 0 until measured
+    bool no_records = false;        // a record partition overflowed: the global table from then on
     bool no_packed = false;      // a packed join table could not place a key: unpacked ones from then on
 };
 
