@@ -218,6 +218,14 @@ bool has_narrow(const tp_table* t) {
     return false;
 }
 
+void lane_drop_arena(tp_engine* e, Lane* lane) {
+    if (!lane->arena) return;
+    cudaFreeAsync(lane->arena, lane->compute);
+    e->arena_total -= lane->arena_bytes;
+    lane->arena = nullptr;
+    lane->arena_bytes = 0;
+}
+
 void dev_free(tp_engine* e, void* p, cudaStream_t st) {
     (void)e;
     if (p) cudaFreeAsync(p, st);
@@ -276,7 +284,7 @@ tp_status tp_init(const tp_config* cfg, tp_engine** out) {
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&e->compute, cudaStreamNonBlocking));
         e->own_compute = true;
     }
-    TP_TRY_CUDA(cudaHostAlloc((void**)&e->host_words, 4096, cudaHostAllocDefault));
+    TP_TRY_CUDA(cudaHostAlloc((void**)&e->host_words, LANE_HOST_BYTES, cudaHostAllocDefault));
     // the page pool: one page-locked allocation cut into equal pages
     PagePool& pp = e->pool;
     pp.page_bytes = e->cfg.page_bytes;
@@ -310,6 +318,7 @@ void tp_shutdown(tp_engine* e) {
     cudaStreamSynchronize(e->compute);
     cudaStreamSynchronize(e->copy);
     cudaStreamSynchronize(e->spill);
+    lane_drop_arena(e, &e->lane0);
     if (e->pool.base) cudaFreeHost(e->pool.base);
     if (e->host_words) cudaFreeHost(e->host_words);
     cudaStreamDestroy(e->copy);

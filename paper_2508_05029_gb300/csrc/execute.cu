@@ -75,23 +75,67 @@ int64_t paged_value(const tp_table* t, int c, uint64_t row) {
     return 0;
 }
 
-// Device memory of one execution, released together at the end.
+// Arenas of an engine's lanes together hold at most this, and an eighth of the
+// device budget.
+constexpr uint64_t ARENA_MAX = 2ull << 30;
+
+// Device memory of one execution, released together at the end.  It comes from
+// the lane's arena while that lasts, then from the stream-ordered allocator;
+// an execution that needed more leaves a larger arena to the next.  Taking
+// every buffer from the allocator cost a small query about 15 us of calls, and
+// next to large results that the caller still held it re-mapped memory for the
+// larger buffers: 1.0 ms in two of three passes of the 15M-group query.
 struct Scratch {
     tp_engine* e;
+    Lane* lane;
     cudaStream_t st;
     std::vector<void*> ptrs;
     uint64_t reserved = 0;
-    explicit Scratch(tp_engine* eng, cudaStream_t s) : e(eng), st(s) {}
+    uint64_t at = 0, total = 0;   // arena bytes handed out, bytes asked for
+    Scratch(tp_engine* eng, Lane* l) : e(eng), lane(l), st(l->compute) {}
     tp_status alloc(void** p, uint64_t bytes) {
+        const uint64_t b = align256(bytes ? bytes : 1);
+        total += b;
+        if (b <= lane->arena_bytes - at) {
+            *p = (uint8_t*)lane->arena + at;
+            at += b;
+            return TP_OK;
+        }
         tp_status s = dev_alloc(e, p, bytes, st);
+        if (s != TP_OK && at == 0 && lane->arena) {   // the arena itself may be what is missing
+            lane_drop_arena(e, lane);
+            cudaStreamSynchronize(st);
+            clear_error();
+            s = dev_alloc(e, p, bytes, st);
+        }
         if (s == TP_OK) ptrs.push_back(*p);
         return s;
+    }
+    // Gives one buffer back early, ordered on stream s; the arena's wait for the end.
+    void drop(void* p, cudaStream_t s) {
+        auto it = std::find(ptrs.begin(), ptrs.end(), p);
+        if (it == ptrs.end()) return;
+        dev_free(e, p, s);
+        ptrs.erase(it);
     }
     void free_all() {
         for (void* p : ptrs) dev_free(e, p, st);
         ptrs.clear();
         if (reserved) release(e, reserved);
         reserved = 0;
+        const uint64_t want = (total + (1ull << 21) - 1) >> 21 << 21;
+        total = at = 0;
+        uint64_t held = 0, cap = 0;
+        if (want <= lane->arena_bytes || tp_budget_query(e, &held, &cap) != TP_OK) return;
+        if (e->arena_total - lane->arena_bytes + want > std::min(ARENA_MAX, cap / 8)) return;
+        lane_drop_arena(e, lane);
+        if (cudaMallocAsync(&lane->arena, want, st) != cudaSuccess) {
+            cudaGetLastError();
+            lane->arena = nullptr;
+            return;
+        }
+        lane->arena_bytes = want;
+        e->arena_total += want;
     }
     ~Scratch() { free_all(); }
 };
@@ -457,9 +501,7 @@ tp_status for_each_batch(ExecState& S, Scratch& sc, F&& kernel) {
         cudaEventDestroy(freed[s]);
         for (int c : S.used) {  // the staging slots go back to the pool after the last kernel
             for (void* p : {slot[s][c], enc[s][c]}) {
-                if (!p) continue;
-                dev_free(e, p, S.lane->compute);
-                sc.ptrs.erase(std::find(sc.ptrs.begin(), sc.ptrs.end(), p));
+                if (p) sc.drop(p, S.lane->compute);
             }
         }
     }
@@ -678,6 +720,83 @@ constexpr uint64_t SEL_SLICE_ROWS = 1ull << 26;
 
 constexpr uint64_t DIRECT_AGG_ALWAYS = 1ull << 20;
 
+// Host copies of every array of r from a copy of its block.
+void take_rows(tp_result* r, const unsigned char* block) {
+    const uint64_t n = r->n_groups;
+    auto at = [&](const void* dev) { return block + ((const unsigned char*)dev - (const unsigned char*)r->dev); };
+    const uint64_t* k = (const uint64_t*)at(r->d_keys);
+    const int64_t* c = (const int64_t*)at(r->d_counts);
+    r->h_keys.assign(k, k + n);
+    r->h_counts.assign(c, c + n);
+    if (n == 0) {   // callers may still ask for a pointer
+        r->h_keys.resize(1);
+        r->h_counts.resize(1);
+    }
+    r->have_keys = r->have_counts = true;
+    uint64_t bytes = 16 * n;
+    for (int s = 0; s < r->n_sum; ++s) {
+        const tp_i128* v = (const tp_i128*)at(r->d_sums[s]);
+        r->h_sums[s].assign(v, v + n);
+        r->h_sums[s].resize(std::max<uint64_t>(n, 1));
+        r->have_sum[s] = true;
+        bytes += 16 * n;
+        if (!r->d_avgs[s]) continue;
+        const double* a = (const double*)at(r->d_avgs[s]);
+        r->h_avgs[s].assign(a, a + n);
+        r->h_avgs[s].resize(std::max<uint64_t>(n, 1));
+        r->have_avg[s] = true;
+        bytes += 8 * n;
+    }
+    r->eng->d2h_bytes += bytes;
+}
+
+// The run-time compiled kernel of one shape: writing the shape out and looking
+// its source up takes longer than a small kernel runs, so a plan remembers its
+// kernels by the values the source is made of.
+template <class F>
+const void* plan_kernel(tp_plan* p, const tpk::QueryDev& q, const int8_t* mode, int kind, const int* narrow,
+                        const tpk::StageGeom& geom, F&& compile) {
+    std::string key;
+    auto put = [&](int v) { key.append((const char*)&v, sizeof(v)); };
+    auto table = [&](const tpk::JoinTable& t) {
+        put(t.direct ? 1 : (t.pay_bits ? 4 : (t.key64 ? 3 : 2)));
+        put(t.part_shift != 0);
+        put(t.lip != nullptr);
+        put(t.many);
+    };
+    put(kind);
+    put(geom.consumers);
+    put(geom.rpl);
+    put(geom.ctas);
+    put(q.has_filter ? 1 + q.fcol.type : 0);
+    put(q.has_join ? 1 + q.fk.type : 0);
+    if (q.has_join) table(q.jt);
+    put(q.n_xjoin);
+    for (int j = 0; j < q.n_xjoin; ++j) {
+        put(q.fkx[j].type);
+        table(q.jtx[j]);
+    }
+    put(q.n_group);
+    for (int g = 0; g < q.n_group; ++g) {
+        put(q.gside[g]);
+        put(q.gside[g] == 0 ? q.gcol[g].type : q.gdim[g]);
+        put(q.gbits[g]);
+    }
+    put(q.n_sum);
+    for (int s = 0; s < q.n_sum; ++s) {
+        put(q.skind[s]);
+        put(q.sa[s].type);
+        put(q.skind[s] == tpk::S_MUL_SUB ? q.sb[s].type : 0);
+        put(mode[s]);
+        put(narrow[s]);
+    }
+    for (auto& k : p->kernels)
+        if (k.first == key) return k.second;
+    const void* k = compile();
+    if (k) p->kernels.emplace_back(key, k);
+    return k;
+}
+
 // ------------------------------------------- partitioned aggregation
 //
 // Records (records.cu) pay when the global table they replace would be
@@ -774,7 +893,11 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     const tpk::QueryDev q = fact_query(S);
     // ---- how evenly the passing rows spread, sampled once per plan
     if (p->rec_skew < 0) {
-        TP_TRY_CUDA(tpk::launch_rec_sample(q, rows, REC_SAMPLES, rec, S.counters, st));
+        void* hist = nullptr;
+        tp_status hs = sc.alloc(&hist, ((uint64_t)rec.n_part + 1) * 4);
+        if (hs) return hs;
+        TP_TRY_CUDA(cudaMemsetAsync(hist, 0, ((uint64_t)rec.n_part + 1) * 4, st));
+        TP_TRY_CUDA(tpk::launch_rec_sample(q, rows, REC_SAMPLES, rec, (uint32_t*)hist, S.counters, st));
         mark_launch(e);
         TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words, S.counters, 16, cudaMemcpyDeviceToHost, st));
         TP_TRY_CUDA(cudaStreamSynchronize(st));
@@ -797,19 +920,18 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     const uint64_t room = align256(std::min(rspan, groups) * (16 + 24 * (uint64_t)ns)) + 4096;
     if (reserve(e, bytes + room)) return NO_RECORDS;
     release(e, room);
-    void* mem = nullptr;
-    tp_status s = dev_alloc(e, &mem, bytes, st);
     struct Held {   // given back on every way out
-        tp_engine* e;
-        void* mem;
+        Scratch& sc;
         uint64_t bytes;
-        cudaStream_t st;
+        void* mem = nullptr;
         ~Held() {
-            dev_free(e, mem, st);
-            release(e, bytes);
+            if (mem) sc.drop(mem, sc.st);
+            release(sc.e, bytes);
         }
-    } held{e, mem, bytes, st};
+    } held{sc, bytes};
+    tp_status s = sc.alloc(&held.mem, bytes);
     if (s) return s;
+    void* mem = held.mem;
     uint8_t* at = (uint8_t*)mem;
     rec.r0 = (uint4*)at;
     at += r0_bytes;
@@ -843,9 +965,11 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
             std::string why;
             const int8_t modes[tpk::MAX_SUM] = {};
             const int narrow[tpk::MAX_SUM] = {};
-            jk = jit_kernel(e, geometry_macros(tpk::JIT_RECORDS_GEOM) +
-                                   shape_struct("JS", q, modes, false, true, narrow) + "#include \"jit_records.cuh\"\n",
-                            "tpj_records", &why);
+            jk = plan_kernel(p, q, modes, -1, narrow, tpk::JIT_RECORDS_GEOM, [&] {
+                return jit_kernel(e, geometry_macros(tpk::JIT_RECORDS_GEOM) +
+                                         shape_struct("JS", q, modes, false, true, narrow) +
+                                         "#include \"jit_records.cuh\"\n", "tpj_records", &why);
+            });
             if (jk) e->jit_launches++;
         }
         s = cuda_check(timer.run(st, rows, [&] {
@@ -1331,10 +1455,7 @@ tp_status part_spill_fact(ExecState& S, Scratch& sc, PartJoin& pj, const tpk::Qu
         for (int c : S.used) part[c] = (const uint8_t*)out[c] + base[p] * (uint64_t)width[c];
         s = append_device_rows(e, pj.fact_spill[p], part, bc[p], sp, false, &enc_w, &enc_base);
     }
-    for (int c : S.used) {  // staging goes back (stream-ordered) once its copies are done
-        dev_free(e, out[c], sp);
-        sc.ptrs.erase(std::find(sc.ptrs.begin(), sc.ptrs.end(), out[c]));
-    }
+    for (int c : S.used) sc.drop(out[c], sp);   // staging goes back (stream-ordered) once its copies are done
     TP_TRY_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
     ce = cudaEventRecord(done, sp);
     if (ce != cudaSuccess) {
@@ -1595,14 +1716,17 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
     }
     const int ns = p->n_sum;
     const float lf = p->load_factor;
-    Scratch sc(e, st);
+    Scratch sc(e, lane);
     // ---- misc words: error word, counters, join side cell
     tp_status s = reserve(e, 4096);
     if (s) return s;
     sc.reserved = 4096;
+    const bool shared = p->strategy == TP_AGG_SHARED;
+    const uint32_t G = shared ? (1u << p->key_bits) : 0;
+    const uint64_t gbytes = (uint64_t)G * (1 + 2 * ns) * 8;   // dense accumulators, zeroed with the misc words
     void* misc = nullptr;
-    if ((s = sc.alloc(&misc, 4096))) return s;
-    TP_TRY_CUDA(cudaMemsetAsync(misc, 0, 4096, st));
+    if ((s = sc.alloc(&misc, 4096 + gbytes))) return s;
+    TP_TRY_CUDA(cudaMemsetAsync(misc, 0, 4096 + gbytes, st));
     S.err = (uint32_t*)misc;
     S.counters = (unsigned long long*)((uint8_t*)misc + 256);
     // ---- filter selectivity from a sample, once per plan (decides eager loads
@@ -1623,8 +1747,6 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             est += n_slots * (align256(max_rows * type_size(S.fact->types[c])) +
                               align256(max_rows * (uint64_t)narrow_width_max(S.fact, c)));
     }
-    const bool shared = p->strategy == TP_AGG_SHARED;
-    const uint32_t G = shared ? (1u << p->key_bits) : 0;
     // many groups under a selective filter: a selection vector of the passing
     // rows' indices, filled and consumed per slice of at most SEL_SLICE_ROWS
     // rows of a batch
@@ -1864,11 +1986,12 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
     tp_result* res = nullptr;
     KernelTimer timer(e);
     if (shared) {
-        void* gacc = nullptr;
-        const uint64_t gbytes = (uint64_t)G * (1 + 2 * ns) * 8;
-        if ((s = sc.alloc(&gacc, gbytes))) return s;
-        TP_TRY_CUDA(cudaMemsetAsync(gacc, 0, gbytes, st));
-        const int grid = tpk::agg_shared_grid(p->key_bits, ns, e->num_sms);
+        void* gacc = (uint8_t*)misc + 4096;
+        int plain_grid = 0;   // asked for only by the plain kernel
+        auto grid = [&] {
+            if (!plain_grid) plain_grid = tpk::agg_shared_grid(p->key_bits, ns, e->num_sms);
+            return plain_grid;
+        };
         const bool want_staged = !(e->cfg.flags & TP_FLAG_NO_STAGED);
         bool fast = want_staged && !(e->cfg.flags & TP_FLAG_EXACT_ONLY) && sums_fit_int64(p, S.fact);
         tpk::TermBounds bounds[tpk::MAX_SUM] = {};
@@ -1916,7 +2039,9 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
                         geom = &tpk::JIT_HASHED_GEOM;
                     if (geom) {
                         std::string why;
-                        jk = jit_kernel(e, dense_shape(q, LJ, *geom, dw, narrow), "tpj_dense", &why);
+                        jk = plan_kernel(S.p, q, LJ.sum_mode, dw, narrow, *geom, [&] {
+                            return jit_kernel(e, dense_shape(q, LJ, *geom, dw, narrow), "tpj_dense", &why);
+                        });
                         if (jk) {
                             L = LJ;   // the ahead-of-time kernel keeps its own layout
                             e->jit_launches++;
@@ -1925,7 +2050,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
                 }
                 if (multi && !jk) {
                     return cuda_check(timer.run(st, rows, [&] {
-                        return tpk::launch_agg_shared(q, rows, (uint64_t*)gacc, p->key_bits, grid, st);
+                        return tpk::launch_agg_shared(q, rows, (uint64_t*)gacc, p->key_bits, grid(), st);
                     }), "aggregate");
                 }
                 // the run-time compiled kernel takes the ragged tail itself
@@ -1940,11 +2065,11 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
                 if (r || whole == rows) return r;
                 mark_launch(e);  // rows after the last whole tile
                 const tpk::QueryDev qt = tpk::offset_rows(q, whole);
-                return cuda_check(tpk::launch_agg_shared(qt, rows - whole, (uint64_t*)gacc, p->key_bits, grid, st),
+                return cuda_check(tpk::launch_agg_shared(qt, rows - whole, (uint64_t*)gacc, p->key_bits, grid(), st),
                                   "aggregate tail");
             }
             return cuda_check(timer.run(st, rows, [&] {
-                return tpk::launch_agg_shared(q, rows, (uint64_t*)gacc, p->key_bits, grid, st);
+                return tpk::launch_agg_shared(q, rows, (uint64_t*)gacc, p->key_bits, grid(), st);
             }), "aggregate");
         };
         auto shared_batch = [&](const tpk::QueryDev& q, uint64_t rows, const std::vector<const void*>& colptr) {
@@ -1965,14 +2090,17 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
         tpk::OutDev od;
         if ((s = alloc_result(e, p, G, &res, &od, S.counters + 1, st))) return s;
         std::unique_ptr<tp_result, void (*)(tp_result*)> guard(res, tp_result_free);
-        TP_TRY_CUDA(tpk::launch_final_dense((const uint64_t*)gacc, p->key_bits, ns, od, st, mode == 2));
+        // a small result's rows come back with the status
+        tpk::HostMirror m{S.err, lane->host_words, (const unsigned char*)res->dev, nullptr};
+        if (res->reserved <= LANE_HOST_BYTES - LANE_WORD_BYTES)
+            m.to = (unsigned char*)lane->host_words + LANE_WORD_BYTES;
+        TP_TRY_CUDA(tpk::launch_final_dense((const uint64_t*)gacc, p->key_bits, ns, od, st, mode == 2, &m));
         mark_launch(e);
-        TP_TRY_CUDA(cudaMemcpyAsync(lane->host_words, misc, 8, cudaMemcpyDeviceToHost, st));
-        TP_TRY_CUDA(cudaMemcpyAsync(lane->host_words + 1, S.counters + 1, 8, cudaMemcpyDeviceToHost, st));
         TP_TRY_CUDA(cudaStreamSynchronize(st));
         e->d2h_bytes += 16;
         if ((s = map_err((uint32_t)lane->host_words[0]))) return s;
         res->n_groups = lane->host_words[1];
+        if (m.to) take_rows(res, m.to);
         timer.collect();
         guard.release();
     } else {
@@ -2015,10 +2143,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
         uint64_t table_reserved = 0;   // reservation held for the current range's table
         double gscale = 1.0;           // growth of the group estimate learned from overflows
         int attempt = 0;
-        auto drop = [&](void* ptr) {
-            dev_free(e, ptr, st);
-            sc.ptrs.erase(std::find(sc.ptrs.begin(), sc.ptrs.end(), ptr));
-        };
+        auto drop = [&](void* ptr) { sc.drop(ptr, st); };
         int n_avg = 0;
         for (int a = 0; a < d.n_agg; ++a) n_avg += d.aggs[a].kind == TP_AGG_AVG;
         const uint64_t row_bytes = 16 + 16 * (uint64_t)ns + 8 * (uint64_t)n_avg;

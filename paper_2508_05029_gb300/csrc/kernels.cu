@@ -273,14 +273,38 @@ cudaError_t launch_agg_global(const QueryDev& q, uint64_t n, const AggTable& t, 
 // ---------------------------------------------------------------- finalise
 
 // One CTA walks the dense table in key order, so the output is sorted.
+// With host words, the same CTA leaves the error word and the group count
+// there, and the rows where the mirror has room for them: page-locked memory
+// the host reads after one synchronisation, in place of a copy per word and
+// per result array.
 __global__ void __launch_bounds__(1024) k_final_dense(const uint64_t* __restrict__ gacc, uint32_t G,
-                                                     int n_sum, const __grid_constant__ OutDev o, int lo_only) {
+                                                     int n_sum, const __grid_constant__ OutDev o, int lo_only,
+                                                     const __grid_constant__ HostMirror m) {
     final_dense_block(gacc, G, n_sum, o, lo_only != 0);
+    if (m.words == nullptr) return;
+    __syncthreads();   // the rows and the count are this CTA's own
+    const uint64_t n = *o.n_groups;
+    if (threadIdx.x == 0) {
+        m.words[0] = *m.err;
+        m.words[1] = n;
+    }
+    if (m.to == nullptr) return;
+    auto copy = [&](const void* a, uint64_t words) {   // arrays of 8-byte words inside the result's block
+        const uint64_t at = ((const unsigned char*)a - m.from) / 8;
+        for (uint64_t i = threadIdx.x; i < words; i += blockDim.x)
+            ((uint64_t*)m.to)[at + i] = ((const uint64_t*)a)[i];
+    };
+    copy(o.keys, n);
+    copy(o.counts, n);
+    for (int s = 0; s < n_sum; ++s) {
+        copy(o.sums[s], 2 * n);
+        if (o.has_avg[s]) copy(o.avgs[s], n);
+    }
 }
 
 cudaError_t launch_final_dense(const uint64_t* gacc, uint32_t key_bits, int n_sum, const OutDev& o,
-                               cudaStream_t st, bool lo_only) {
-    k_final_dense<<<1, 1024, 0, st>>>(gacc, 1u << key_bits, n_sum, o, lo_only ? 1 : 0);
+                               cudaStream_t st, bool lo_only, const HostMirror* m) {
+    k_final_dense<<<1, 1024, 0, st>>>(gacc, 1u << key_bits, n_sum, o, lo_only ? 1 : 0, m ? *m : HostMirror{});
     return cudaGetLastError();
 }
 

@@ -400,8 +400,15 @@ cudaError_t launch_agg_global(const QueryDev& q, uint64_t n, const AggTable& t, 
                               cudaStream_t st);
 // lo_only: the table's sums were accumulated as 64-bit values (overflow ruled
 // out by column bounds); their high words are the sign extension of the low.
+// m: where the host reads the status and the rows (nullptr: nowhere).
+struct HostMirror {
+    const uint32_t* err;        // error word
+    uint64_t* words;            // host: error word, group count
+    const unsigned char* from;  // the result's block
+    unsigned char* to;          // host: its copy (nullptr: rows stay on the device)
+};
 cudaError_t launch_final_dense(const uint64_t* gacc, uint32_t key_bits, int n_sum, const OutDev& o,
-                               cudaStream_t st, bool lo_only = false);
+                               cudaStream_t st, bool lo_only = false, const HostMirror* m = nullptr);
 // Loads the build, plain shared-memory aggregation and dense finalisation
 // kernels on the current device now (with lazy module loading the first
 // launch would load them, placing their code in device memory then).
@@ -470,9 +477,9 @@ uint32_t rec_direct_smem(int shift, int n_sum);
 cudaError_t launch_rec_emit(const RecDev& rec, int n_sum, const uint32_t* groups, const unsigned long long* offsets,
                             const OutDev& o, int num_sms, cudaStream_t st);
 // Of `samples` evenly spaced rows: out[0] = those passing the filter, out[1] =
-// the most of them in one partition.
+// the most of them in one partition; hist: n_part + 1 zeroed words.
 cudaError_t launch_rec_sample(const QueryDev& q, uint64_t n, uint32_t samples, const RecDev& rec,
-                              unsigned long long* out, cudaStream_t st);
+                              uint32_t* hist, unsigned long long* out, cudaStream_t st);
 // HyperLogLog registers (HLL_REGS words, zeroed) of the rows' group keys.
 cudaError_t launch_rec_distinct(const QueryDev& q, uint64_t n, uint32_t* regs, int num_sms, cudaStream_t st);
 

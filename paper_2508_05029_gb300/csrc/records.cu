@@ -460,20 +460,17 @@ __global__ void __launch_bounds__(256) k_rec_emit(const __grid_constant__ RecDev
     }
 }
 
-// How evenly samples of the passing rows spread over the partitions: out[0] =
-// samples passing the filter, out[1] = most in one partition.  One CTA.
-constexpr int RSAMPLE_THREADS = 1024;
+// How evenly samples of the passing rows spread over the partitions: hist
+// (n_part + 1 zeroed words) counts them, and the CTA that ends last writes
+// out[0] = samples passing the filter, out[1] = most in one partition.
+constexpr int RSAMPLE_THREADS = 256;
 __global__ void __launch_bounds__(RSAMPLE_THREADS)
     k_rec_sample(const __grid_constant__ QueryDev q, uint64_t n, uint32_t samples, const __grid_constant__ RecDev rec,
-                 unsigned long long* out) {
-    extern __shared__ uint32_t rsm[];
+                 uint32_t* hist, unsigned long long* out) {
     __shared__ uint32_t most, passed;
-    for (uint32_t p = threadIdx.x; p < rec.n_part; p += RSAMPLE_THREADS) rsm[p] = 0;
+    __shared__ bool last;
     if (threadIdx.x == 0) most = passed = 0;
-    __syncthreads();
-    uint32_t mine = 0;
-#pragma unroll 8
-    for (uint32_t j = threadIdx.x; j < samples; j += RSAMPLE_THREADS) {
+    for (uint32_t j = blockIdx.x * RSAMPLE_THREADS + threadIdx.x; j < samples; j += gridDim.x * RSAMPLE_THREADS) {
         const uint64_t r = (uint64_t)(((unsigned __int128)j * n) / samples);
         if (q.has_filter) {
             const int64_t v = ld1(q.fcol, r);
@@ -484,13 +481,23 @@ __global__ void __launch_bounds__(RSAMPLE_THREADS)
             const uint64_t f = (uint64_t)ld1(q.gcol[g], r);
             key = q.gbits[g] < 64 ? key << q.gbits[g] | f : f;
         }
-        ++mine;
         key -= rec.kmin;
-        if (key < rec.span) atomicAdd(&rsm[key >> rec.shift], 1u);
+        if (key < rec.span) atomicAdd(&hist[key >> rec.shift], 1u);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&hist[rec.n_part], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    uint32_t mine = 0, top = 0;
+    for (uint32_t p = threadIdx.x; p < rec.n_part; p += RSAMPLE_THREADS) {
+        const uint32_t c = __ldcg(hist + p);
+        mine += c;
+        top = max(top, c);
     }
     atomicAdd(&passed, mine);
-    __syncthreads();
-    for (uint32_t p = threadIdx.x; p < rec.n_part; p += RSAMPLE_THREADS) atomicMax(&most, rsm[p]);
+    atomicMax(&most, top);
     __syncthreads();
     if (threadIdx.x == 0) {
         out[0] = passed;
@@ -633,8 +640,9 @@ cudaError_t launch_rec_emit(const RecDev& rec, int n_sum, const uint32_t* groups
 }
 
 cudaError_t launch_rec_sample(const QueryDev& q, uint64_t n, uint32_t samples, const RecDev& rec,
-                              unsigned long long* out, cudaStream_t st) {
-    k_rec_sample<<<1, RSAMPLE_THREADS, 4 * rec.n_part, st>>>(q, n, samples, rec, out);
+                              uint32_t* hist, unsigned long long* out, cudaStream_t st) {
+    const unsigned grid = (samples + RSAMPLE_THREADS - 1) / RSAMPLE_THREADS;
+    k_rec_sample<<<std::min(grid, 256u), RSAMPLE_THREADS, 0, st>>>(q, n, samples, rec, hist, out);
     return cudaGetLastError();
 }
 

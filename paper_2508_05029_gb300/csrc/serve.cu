@@ -762,6 +762,7 @@ void server_free(tp_server* sv) {
     cache_evict_idle(sv->e, &sv->cache, 0);
     evict_joins(sv, 0, sv->e->compute);
     for (Lane& l : sv->lanes) {
+        lane_drop_arena(sv->e, &l);
         if (l.compute) cudaStreamDestroy(l.compute);
         if (l.copy) cudaStreamDestroy(l.copy);
         if (l.spill) cudaStreamDestroy(l.spill);
@@ -797,13 +798,13 @@ tp_status tp_server_start(tp_engine* e, int32_t workers, int32_t max_inflight, u
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&l.compute, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&l.copy, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&l.spill, cudaStreamNonBlocking));
-        TP_TRY_CUDA(cudaHostAlloc((void**)&l.host_words, 4096, cudaHostAllocDefault));
+        TP_TRY_CUDA(cudaHostAlloc((void**)&l.host_words, LANE_HOST_BYTES, cudaHostAllocDefault));
     }
     if (sv->batch_on) {
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&sv->dlane.compute, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&sv->dlane.copy, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&sv->dlane.spill, cudaStreamNonBlocking));
-        TP_TRY_CUDA(cudaHostAlloc((void**)&sv->dlane.host_words, 4096, cudaHostAllocDefault));
+        TP_TRY_CUDA(cudaHostAlloc((void**)&sv->dlane.host_words, LANE_HOST_BYTES, cudaHostAllocDefault));
         for (Slot& sl : sv->slots) {
             TP_TRY_CUDA(cudaStreamCreateWithFlags(&sl.st, cudaStreamNonBlocking));
             TP_TRY_CUDA(cudaEventCreateWithFlags(&sl.ev, cudaEventDisableTiming));

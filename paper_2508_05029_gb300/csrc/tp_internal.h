@@ -99,8 +99,14 @@ struct Lane {
     cudaStream_t compute = nullptr;
     cudaStream_t copy = nullptr;      // host -> device prefetch
     cudaStream_t spill = nullptr;     // device -> host spill copies (the other link direction)
-    uint64_t* host_words = nullptr;   // 4 KB pinned
+    uint64_t* host_words = nullptr;   // LANE_HOST_BYTES pinned: status words, then a small result's rows
+    // device memory kept between the lane's executions for their scratch
+    // (stream-ordered on compute: an execution starts after the one before)
+    void* arena = nullptr;
+    uint64_t arena_bytes = 0;
 };
+constexpr uint64_t LANE_WORD_BYTES = 4096;
+constexpr uint64_t LANE_HOST_BYTES = LANE_WORD_BYTES + (128u << 10);
 
 }  // namespace tp
 
@@ -121,6 +127,7 @@ struct tp_engine {
     std::atomic<uint64_t> h2d_bytes{0}, d2h_bytes{0}, batches{0}, launches{0}, retries{0};
     std::atomic<uint64_t> jit_compiles{0}, jit_failures{0}, jit_launches{0}, jit_us{0};
     std::atomic<uint64_t> split_passes{0}, lip_filters{0};
+    std::atomic<uint64_t> arena_total{0};   // bytes of all lanes' arenas
     // small pinned scratch for status words read back after an execution
     uint64_t* host_words = nullptr;
     tp::Lane lane0;                  // compute, copy, host_words of the engine itself
@@ -177,6 +184,8 @@ struct tp_plan {
     uint64_t distinct_groups = 0;   // estimated distinct group keys of the fact table, 0 until measured
     double rec_skew = -1.0;         // sampled: fullest key partition over the mean, < 0 until measured
     bool no_records = false;        // a record partition overflowed: the global table from then on
+    // run-time compiled kernels by the bytes of their shape and geometry
+    std::vector<std::pair<std::string, const void*>> kernels;
     bool no_packed = false;      // a packed join table could not place a key: unpacked ones from then on
 };
 
@@ -345,6 +354,8 @@ int batch_kernel_grid(const void* jit_kernel_or_null, uint32_t smem_bytes, int n
 tp_status alloc_result(tp_engine* e, tp_plan* p, uint64_t cap, tp_result** out, tpk::OutDev* od,
                        unsigned long long* n_groups_dev, cudaStream_t st);
 
+// Gives a lane's arena back (its work has finished or is ordered before).
+void lane_drop_arena(tp_engine* e, Lane* lane);
 // device memory (stream-ordered allocator on the compute stream)
 tp_status dev_alloc(tp_engine* e, void** p, uint64_t bytes, cudaStream_t st);
 void dev_free(tp_engine* e, void* p, cudaStream_t st);

@@ -524,8 +524,9 @@ class Result:
     def _arr(self, ptr, dtype, n):
         if not ptr:
             raise TPError(TP_E_CUDA, last_error())
-        return np.ctypeslib.as_array(ctypes.cast(ptr, ctypes.POINTER(np.ctypeslib.as_ctypes_type(dtype))),
-                                     shape=(max(n, 1),))[:n].copy()
+        out = np.empty(n, dtype)
+        ctypes.memmove(out.ctypes.data, ptr, out.nbytes)
+        return out
 
     def keys(self) -> np.ndarray:
         return self._arr(self.eng.lib.tp_result_keys(self.h), np.uint64, self.n_groups)
@@ -539,8 +540,9 @@ class Result:
         p = self.eng.lib.tp_result_sum(self.h, agg)
         if not p:
             raise TPError(TP_E_INVALID, last_error() or f"aggregate {agg} has no sum")
-        raw = np.ctypeslib.as_array(ctypes.cast(p, ctypes.POINTER(ctypes.c_uint64)), shape=(max(n, 1) * 2,))
-        return raw[: 2 * n].copy().reshape(n, 2)
+        out = np.empty((n, 2), np.uint64)
+        ctypes.memmove(out.ctypes.data, p, out.nbytes)
+        return out
 
     def avg(self, agg: int) -> np.ndarray:
         return self._arr(self.eng.lib.tp_result_avg(self.h, agg), np.float64, self.n_groups)
