@@ -117,40 +117,42 @@ __device__ __forceinline__ void atomic_add_i128(uint64_t* lo, uint64_t* hi, I128
 // Lookahead information passing (Section 5): the keys of the dimension rows
 // that pass the dimension predicate go into a blocked Bloom filter, and fact
 // rows test their key before the probe (and before a partitioned join spills
-// them).  With h = fmix64(key), the top bits of h pick one 256-bit block (an
-// aligned 32-byte sector) and word w of the block holds bit
-// (lo32(h) * M_w) >> 27 with the odd multiplier M_w = 0x9E3779B1 * (2w + 1).
-// A test reads one sector; an inserted key always passes.
+// them).  With h = fmix64(key), the top bits of h pick one 64-bit word and its
+// low 20 bits two bits in each half of the word.  An insert is one reduction
+// and a test one 8-byte load; at 16 bits per key about one key in 500 passes
+// that was not inserted, and an inserted key always does.  (Eight 32-bit words
+// of 256-bit blocks: eight reductions per insert, two 16-byte loads and twice
+// the instructions per test.)
 
-__device__ __forceinline__ uint32_t lip_bit(uint32_t h, uint32_t w) {
-    return 1u << ((h * (0x9E3779B1u * (2u * w + 1u))) >> 27);
+__device__ __forceinline__ uint64_t lip_bits(uint32_t h) {
+    const uint32_t lo = 1u << (h & 31u) | 1u << (h >> 5 & 31u), hi = 1u << (h >> 10 & 31u) | 1u << (h >> 15 & 31u);
+    return (uint64_t)hi << 32 | lo;
 }
 
 __device__ __forceinline__ bool lip_test(const JoinTable& jt, int64_t key) {
     const uint64_t h = fmix64((uint64_t)key);
-    const uint4* blk = reinterpret_cast<const uint4*>(jt.lip + ((h >> jt.lip_shift) << 3));
-    const uint4 a = __ldg(blk), b = __ldg(blk + 1);
-    const uint32_t l = (uint32_t)h;
-    const uint32_t miss = (~a.x & lip_bit(l, 0)) | (~a.y & lip_bit(l, 1)) | (~a.z & lip_bit(l, 2)) |
-                          (~a.w & lip_bit(l, 3)) | (~b.x & lip_bit(l, 4)) | (~b.y & lip_bit(l, 5)) |
-                          (~b.z & lip_bit(l, 6)) | (~b.w & lip_bit(l, 7));
-    return miss == 0;
+    return (~__ldg((const unsigned long long*)jt.lip + (h >> jt.lip_shift)) & lip_bits((uint32_t)h)) == 0;
 }
 
 __device__ __forceinline__ void lip_insert(const JoinTable& jt, int64_t key) {
     const uint64_t h = fmix64((uint64_t)key);
-    uint32_t* blk = jt.lip + ((h >> jt.lip_shift) << 3);
-#pragma unroll
-    for (uint32_t w = 0; w < 8; ++w) atomicOr(blk + w, lip_bit((uint32_t)h, w));
+    atomicOr((unsigned long long*)jt.lip + (h >> jt.lip_shift), (unsigned long long)lip_bits((uint32_t)h));
 }
 
 // Clears bit j of pm for rows whose key the lookahead filter rules out.
 template <int N>
 __device__ __forceinline__ void lip_mask(const JoinTable& jt, const int64_t* key, uint32_t& pm) {
     if (jt.lip == nullptr) return;
+    uint64_t miss[N];   // the rows' words in flight together
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const uint64_t h = fmix64((uint64_t)key[j]);
+        miss[j] = lip_bits((uint32_t)h);
+        if ((pm >> j) & 1u) miss[j] &= ~__ldg((const unsigned long long*)jt.lip + (h >> jt.lip_shift));
+    }
 #pragma unroll
     for (int j = 0; j < N; ++j)
-        if (((pm >> j) & 1u) && !lip_test(jt, key[j])) pm &= ~(1u << j);
+        if (miss[j] != 0) pm &= ~(1u << j);
 }
 
 // Does dimension row i pass the dimension predicate?
@@ -574,22 +576,23 @@ __device__ __forceinline__ void final_dense_block(const uint64_t* __restrict__ g
 
 // ------------------------------------------------------------- join build
 
-// Inserts dimension row i into the join table: CAS on the key (32-bit keys:
-// key and payload in one word), ERR_DUP on a repeated key.
-__device__ __forceinline__ void build_insert(const BuildDev& b, uint64_t i) {
-    const JoinTable& jt = b.jt;
-    if (!dim_row_admitted(b, i)) return;
-    int64_t key = ld1(b.key, i);
-    if (jt.lip != nullptr) lip_insert(jt, key);
-    // Dimension group fields packed into bits 0..30 of the payload; bit 31
-    // marks a row with a field outside its width.  That is an error only
-    // if a surviving fact row joins to it, which the probe side reports.
+// Dimension row i's group fields packed into bits 0..30 of its payload; bit 31
+// marks a row with a field outside its width.  That is an error only if a
+// surviving fact row joins to it, which the probe side reports.
+__device__ __forceinline__ uint32_t build_payload(const BuildDev& b, uint64_t i) {
     uint32_t payload = 0;
     for (int f = 0; f < b.n_dfield; ++f) {
         int64_t v = ld1(b.dcol[f], i);
         if (v < 0 || ((uint64_t)v >> b.dbits[f]) != 0) payload |= PAYLOAD_BAD;
         else payload |= (uint32_t)((uint64_t)v << b.dpos[f]);
     }
+    return payload;
+}
+
+// Inserts (key, payload) into the join table: CAS on the key (32-bit keys: key
+// and payload in one word), ERR_DUP on a repeated key.
+__device__ __forceinline__ void build_insert_key(const BuildDev& b, int64_t key, uint32_t payload) {
+    const JoinTable& jt = b.jt;
     if (jt.direct) {  // slot key - kmin: the host sized the table to the key range
         const uint32_t v = (payload & PAYLOAD_BAD) ? PAYLOAD_BAD : payload;
         const uint64_t idx = (uint64_t)key - (uint64_t)jt.kmin;
@@ -604,7 +607,17 @@ __device__ __forceinline__ void build_insert(const BuildDev& b, uint64_t i) {
         const uint64_t pay = (payload & PAYLOAD_BAD) ? 1ull << (jt.pay_bits - 1) : (uint64_t)payload;
         for (uint32_t dist = 0; dist <= PACK_MAX_DIST; ++dist) {
             unsigned long long* bucket = (unsigned long long*)jt.slots + 4 * (uint64_t)at;
-            for (int m = 0; m < 4; ++m) {
+            // the words seen taken need no compare-and-swap of their own
+            const ulonglong2 x = __ldcg((const ulonglong2*)bucket), y = __ldcg((const ulonglong2*)bucket + 1);
+            const uint64_t w[4] = {x.x, x.y, y.x, y.y};
+            int m = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (m != k || w[k] == EMPTY64) continue;
+                if ((w[k] ^ word) >> jt.pay_bits == 0) { atomicOr(b.err, ERR_DUP); return; }
+                m = k + 1;
+            }
+            for (; m < 4; ++m) {
                 const unsigned long long prev =
                     atomicCAS(bucket + m, (unsigned long long)EMPTY64, (unsigned long long)(word | pay));
                 if (prev == EMPTY64) return;
@@ -646,6 +659,18 @@ __device__ __forceinline__ void build_insert(const BuildDev& b, uint64_t i) {
         s = (s + 1) & jt.mask;
     }
     if (!placed) atomicOr(b.err, ERR_INTERNAL);
+}
+
+// Inserts dimension row i, which the predicate admits, and its key into the
+// lookahead filter; build_insert: if the predicate admits it.
+__device__ __forceinline__ void build_insert_row(const BuildDev& b, uint64_t i) {
+    const int64_t key = ld1(b.key, i);
+    if (b.jt.lip != nullptr) lip_insert(b.jt, key);
+    build_insert_key(b, key, build_payload(b, i));
+}
+
+__device__ __forceinline__ void build_insert(const BuildDev& b, uint64_t i) {
+    if (dim_row_admitted(b, i)) build_insert_row(b, i);
 }
 
 // ------------------------------------------------------- global aggregation slot

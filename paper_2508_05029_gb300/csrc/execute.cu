@@ -1916,7 +1916,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             int lg = 0;
             while ((1ull << lg) < lip_blocks) ++lg;
             S.jt.lip = (uint32_t*)lip;
-            S.jt.lip_shift = 64 - lg;
+            S.jt.lip_shift = 62 - lg;   // four words per 32 bytes
             e->lip_filters++;
         } else {
             clear_error();
@@ -1977,7 +1977,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             int lg = 0;
             while ((1ull << lg) < x.lip_blocks) ++lg;
             jt.lip = (uint32_t*)lip;
-            jt.lip_shift = 64 - lg;
+            jt.lip_shift = 62 - lg;   // four words per 32 bytes
             e->lip_filters++;
         }
         if ((s = build_join(S, sc, 1 + j))) return s;

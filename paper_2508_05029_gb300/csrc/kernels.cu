@@ -67,18 +67,55 @@ cudaError_t launch_init_agg(uint64_t* slots, uint64_t n_slots, uint32_t words, c
 
 // -------------------------------------------------------------------- build
 
-__global__ void __launch_bounds__(256) k_build(const __grid_constant__ BuildDev b, uint64_t n) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        build_insert(b, i);
+// A row is a chain of dependent accesses (key and fields, table), hidden by
+// the SM's 64 warps.  Under a predicate a CTA first lists its tile's admitted
+// rows, so every lane of the chain has one: 32M rows, 12% of them admitted,
+// took 321 us when lanes of refused rows waited beside them, 195 now.
+// (Four rows per thread in lock step, with a third of the warps: 953 us.)
+constexpr int BUILD_THREADS = 256;
+constexpr int BUILD_CHECK = 8;   // rows per thread checked per tile
+
+__global__ void __launch_bounds__(BUILD_THREADS, 8) k_build(const __grid_constant__ BuildDev b, uint64_t n) {
+    if (!b.has_filter) {
+        for (uint64_t i = blockIdx.x * (uint64_t)BUILD_THREADS + threadIdx.x; i < n;
+             i += (uint64_t)gridDim.x * BUILD_THREADS)
+            build_insert_row(b, i);
+        return;
+    }
+    constexpr uint32_t TILE = BUILD_THREADS * BUILD_CHECK;
+    __shared__ uint16_t list[TILE];
+    __shared__ uint32_t count;
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * TILE; t0 < n; t0 += (uint64_t)gridDim.x * TILE) {
+        if (threadIdx.x == 0) count = 0;
+        int64_t v[BUILD_CHECK];
+#pragma unroll
+        for (int u = 0; u < BUILD_CHECK; ++u) {
+            const uint64_t i = t0 + u * BUILD_THREADS + threadIdx.x;
+            v[u] = i < n ? ld1(b.fcol, i) : 0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < BUILD_CHECK; ++u) {
+            const uint32_t r = u * BUILD_THREADS + threadIdx.x;
+            const bool on = t0 + r < n && v[u] >= b.flo && v[u] <= b.fhi;
+            const unsigned m = __ballot_sync(0xffffffffu, on);
+            uint32_t at = 0;
+            if (m != 0 && lane == 0) at = atomicAdd(&count, (uint32_t)__popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (on) list[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)r;
+        }
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < count; i += BUILD_THREADS) build_insert_row(b, t0 + list[i]);
+        __syncthreads();
+    }
 }
 
 cudaError_t launch_build(const BuildDev& b, uint64_t n, int num_sms, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    uint64_t blocks = (n + 255) / 256;
-    uint64_t cap = (uint64_t)num_sms * 8;
-    if (blocks > cap) blocks = cap;
-    k_build<<<(unsigned)blocks, 256, 0, st>>>(b, n);
+    const uint64_t tile = b.has_filter ? BUILD_THREADS * BUILD_CHECK : BUILD_THREADS;
+    const uint64_t blocks = std::min<uint64_t>((n + tile - 1) / tile, (uint64_t)num_sms * 8);   // one wave
+    k_build<<<(unsigned)blocks, BUILD_THREADS, 0, st>>>(b, n);
     return cudaGetLastError();
 }
 

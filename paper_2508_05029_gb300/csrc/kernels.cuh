@@ -90,7 +90,7 @@ struct JoinTable {
     int32_t part_shift;
     int32_t cap_bits;       // packed hash: log2(buckets)
     // lookahead filter (lip != nullptr): a blocked Bloom filter of the
-    // admitted build keys, 8 words per block; a key's block is
+    // admitted build keys in 64-bit words; a key's word is
     // fmix64(key) >> lip_shift
     uint32_t* lip;
     int32_t lip_shift;
