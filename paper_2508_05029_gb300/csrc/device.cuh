@@ -139,17 +139,24 @@ __device__ __forceinline__ void lip_insert(const JoinTable& jt, int64_t key) {
     atomicOr((unsigned long long*)jt.lip + (h >> jt.lip_shift), (unsigned long long)lip_bits((uint32_t)h));
 }
 
-// Clears bit j of pm for rows whose key the lookahead filter rules out.
+// miss[j] != 0: the lookahead filter rules row j's key out (rows of pm; the
+// rows' words are in flight together, and may stay so while others load).
 template <int N>
-__device__ __forceinline__ void lip_mask(const JoinTable& jt, const int64_t* key, uint32_t& pm) {
-    if (jt.lip == nullptr) return;
-    uint64_t miss[N];   // the rows' words in flight together
+__device__ __forceinline__ void lip_load(const JoinTable& jt, const int64_t* key, uint32_t pm, uint64_t miss[N]) {
 #pragma unroll
     for (int j = 0; j < N; ++j) {
         const uint64_t h = fmix64((uint64_t)key[j]);
         miss[j] = lip_bits((uint32_t)h);
         if ((pm >> j) & 1u) miss[j] &= ~__ldg((const unsigned long long*)jt.lip + (h >> jt.lip_shift));
     }
+}
+
+// Clears bit j of pm for rows whose key the lookahead filter rules out.
+template <int N>
+__device__ __forceinline__ void lip_mask(const JoinTable& jt, const int64_t* key, uint32_t& pm) {
+    if (jt.lip == nullptr) return;
+    uint64_t miss[N];
+    lip_load<N>(jt, key, pm, miss);
 #pragma unroll
     for (int j = 0; j < N; ++j)
         if (miss[j] != 0) pm &= ~(1u << j);

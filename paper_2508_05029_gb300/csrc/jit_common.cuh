@@ -291,15 +291,37 @@ __device__ __forceinline__ void accumulate(const QueryDev& q, const Tab& t, cons
 // Star join: further join J (and the following ones) of the rows in pm --
 // lookahead filter, probe of its own table, payload into pays[1 + J]; rows
 // without a partner leave pm.
+// The filters' words are loaded beside the first join's probe (miss[J]), which
+// takes one of the row's three dependent accesses away: 786 -> 737 us for 60M
+// rows joined to a direct and a filtered hashed table.
+template <class S, int J, class C>
+__device__ __forceinline__ void further_lips(const QueryDev& q, const C& c, uint32_t r0, uint32_t pm,
+                                             uint64_t (&miss)[MAX_XJOIN][ST_RPL]) {
+    if constexpr (J < S::nx) {
+        if constexpr (S::xlip[J]) {
+            int64_t key[ST_RPL];
+#pragma unroll
+            for (int j = 0; j < ST_RPL; ++j) key[j] = (int64_t)c.template ld<S::xktype[J], CI_X + J>(r0, j);
+            lip_load<ST_RPL>(q.jtx[J], key, pm, miss[J]);
+        }
+        further_lips<S, J + 1, C>(q, c, r0, pm, miss);
+    }
+}
+
 template <class S, int J, class C>
 __device__ __forceinline__ void further_joins(const QueryDev& q, const C& c, uint32_t r0,
+                                              const uint64_t (&miss)[MAX_XJOIN][ST_RPL],
                                               uint32_t (&pays)[1 + MAX_XJOIN][ST_RPL], uint32_t& pm) {
     if constexpr (J < S::nx) {
         const JoinTable& jt = q.jtx[J];
         int64_t key[ST_RPL];
 #pragma unroll
         for (int j = 0; j < ST_RPL; ++j) key[j] = (int64_t)c.template ld<S::xktype[J], CI_X + J>(r0, j);
-        if constexpr (S::xlip[J]) lip_mask<ST_RPL>(jt, key, pm);
+        if constexpr (S::xlip[J]) {
+#pragma unroll
+            for (int j = 0; j < ST_RPL; ++j)
+                if (miss[J][j] != 0) pm &= ~(1u << j);
+        }
         uint32_t* pay = pays[1 + J];
         if constexpr (S::xjoin[J] == J_DIRECT) {
 #pragma unroll
@@ -325,7 +347,7 @@ __device__ __forceinline__ void further_joins(const QueryDev& q, const C& c, uin
             pm &= ~bad;
         }
         if (!pm) return;
-        further_joins<S, J + 1, C>(q, c, r0, pays, pm);
+        further_joins<S, J + 1, C>(q, c, r0, miss, pays, pm);
     }
 }
 
@@ -361,6 +383,8 @@ __device__ __forceinline__ void consume(const QueryDev& q, const Flt& flt, const
         lip_mask<ST_RPL>(q.jt, key, pm);
         if (!pm) return;
     }
+    uint64_t miss[MAX_XJOIN][ST_RPL];
+    if constexpr (S::nx > 0) further_lips<S, 0, C>(q, c, r0, pm, miss);
     if constexpr (S::join == J_DIRECT) {
         const unsigned int* dt = (const unsigned int*)q.jt.slots;
 #pragma unroll
@@ -395,7 +419,7 @@ __device__ __forceinline__ void consume(const QueryDev& q, const Flt& flt, const
         if (!pm) return;
     }
     if constexpr (S::nx > 0) {
-        further_joins<S, 0, C>(q, c, r0, pays, pm);
+        further_joins<S, 0, C>(q, c, r0, miss, pays, pm);
         if (!pm) return;
     }
     if constexpr (S::many) {
