@@ -1052,8 +1052,13 @@ uint64_t agg_table_bytes(bool direct, uint64_t span, uint64_t cap, uint32_t word
 // spills (each holds a staging buffer).
 constexpr size_t SPILL_BACKLOG = 2;
 
+// Where in a lane's host words a fact batch's partition counts arrive.
+constexpr int PART_WORDS = 64;
+
 struct PartJoin {
     bool on = false;
+    cudaStream_t build_stream = nullptr;   // carries the build side's spill copies
+    cudaEvent_t counted = nullptr;         // a fact batch's partition counts have arrived
     int P = 0;
     int shift = 0;
     uint64_t spill_mask = 0;               // partitions not resident
@@ -1085,6 +1090,8 @@ struct PartJoin {
     std::vector<int64_t> enc_base;
     std::vector<int> width;
     ~PartJoin() {
+        if (build_stream) cudaStreamSynchronize(build_stream);   // a failed execution: copies into the pages given back
+        if (counted) cudaEventDestroy(counted);
         for (cudaEvent_t ev : inflight) {
             cudaEventSynchronize(ev);
             cudaEventDestroy(ev);
@@ -1172,28 +1179,38 @@ tp_status part_setup(ExecState& S, Scratch& sc, PartJoin& pj, uint64_t table_bud
     tp_engine* e = S.e;
     cudaStream_t st = S.lane->compute;
     const int P = pj.P;
+    // counts and cursors of the fact batches, then of every build batch (its
+    // counts, which become its bases, and its cursors): the build batches are
+    // counted in one pass, so the scatter pass knows every batch's shares and
+    // waits for nothing
+    const uint64_t nb = S.dim->placement == PL_PAGES ? std::max<uint64_t>(1, S.dim->batches.size()) : 1;
     void* words = nullptr;
-    tp_status s = sc.alloc(&words, 2 * 8 * (uint64_t)P);
+    tp_status s = sc.alloc(&words, 2 * 8 * (uint64_t)P * (1 + nb));
     if (s) return s;
     pj.counts = (unsigned long long*)words;
     pj.cursor = pj.counts + P;
-    TP_TRY_CUDA(cudaMemsetAsync(pj.counts, 0, 8 * (uint64_t)P, st));
+    unsigned long long* bcounts = pj.counts + 2 * P;
+    unsigned long long* bcursor = bcounts + nb * P;
+    TP_TRY_CUDA(cudaMemsetAsync(words, 0, 2 * 8 * (uint64_t)P * (1 + nb), st));
     const uint64_t slot = S.key64 ? 16 : 8;
     auto table_bytes = [&](uint64_t rows) {
         return pow2_at_least(std::max<uint64_t>(64, (uint64_t)std::ceil(rows / lf))) * slot;
     };
     // the per-partition counts decide residency only when not every build
     // row fits: otherwise the histogram pass over the build side is skipped
-    std::vector<unsigned long long> cnt(P, 0);
+    std::vector<unsigned long long> cnt(P, 0), bc(nb * P, 0);
     if (table_bytes(S.dim->rows) > table_budget) {
+        uint64_t bi = 0;
         s = for_each_dim_batch(S, sc, proto, [&](const tpk::BuildDev& b, uint64_t rows) {
             mark_launch(e);
-            return cuda_check(tpk::launch_part_hist(b, rows, pj.shift, pj.counts, e->num_sms, st),
+            return cuda_check(tpk::launch_part_hist(b, rows, pj.shift, bcounts + P * bi++, e->num_sms, st),
                               "partition");
         });
         if (s) return s;
-        TP_TRY_CUDA(cudaMemcpyAsync(cnt.data(), pj.counts, 8 * (uint64_t)P, cudaMemcpyDeviceToHost, st));
+        TP_TRY_CUDA(cudaMemcpyAsync(bc.data(), bcounts, 8 * nb * P, cudaMemcpyDeviceToHost, st));
         TP_TRY_CUDA(cudaStreamSynchronize(st));
+        for (uint64_t k = 0; k < nb; ++k)
+            for (int p = 0; p < P; ++p) cnt[p] += bc[k * P + p];
     } else {
         cnt[0] = S.dim->rows;   // only the total matters below
     }
@@ -1246,32 +1263,33 @@ tp_status part_setup(ExecState& S, Scratch& sc, PartJoin& pj, uint64_t table_bud
     if (pj.spill_mask) {
         if ((s = sc.alloc(&skeys, align256(max_rows * 8))) || (s = sc.alloc(&spays, align256(max_rows * 4)))) return s;
     }
-    return for_each_dim_batch(S, sc, proto, [&](const tpk::BuildDev& b, uint64_t rows) -> tp_status {
-        mark_launch(e);
-        if (!pj.spill_mask) return cuda_check(tpk::launch_build(b, rows, e->num_sms, st), "build");
-        TP_TRY_CUDA(cudaMemsetAsync(pj.counts, 0, 2 * 8 * (uint64_t)P, st));
-        TP_TRY_CUDA(tpk::launch_part_hist(b, rows, pj.shift, pj.counts, e->num_sms, st));
-        std::vector<unsigned long long> bc(P), base(P, 0);
-        TP_TRY_CUDA(cudaMemcpyAsync(bc.data(), pj.counts, 8 * (uint64_t)P, cudaMemcpyDeviceToHost, st));
-        TP_TRY_CUDA(cudaStreamSynchronize(st));
+    std::vector<unsigned long long> base(nb * P, 0);
+    for (uint64_t k = 0; k < nb; ++k) {
         uint64_t run = 0;
         for (int p = 0; p < P; ++p) {
-            base[p] = run;
-            if ((pj.spill_mask >> p) & 1ull) run += bc[p];
+            base[k * P + p] = run;
+            if ((pj.spill_mask >> p) & 1ull) run += bc[k * P + p];
         }
-        TP_TRY_CUDA(cudaMemcpyAsync(pj.counts, base.data(), 8 * (uint64_t)P, cudaMemcpyHostToDevice, st));
+    }
+    pj.build_stream = st;
+    if (pj.spill_mask) TP_TRY_CUDA(cudaMemcpyAsync(bcounts, base.data(), 8 * nb * P, cudaMemcpyHostToDevice, st));
+    uint64_t bi = 0;
+    s = for_each_dim_batch(S, sc, proto, [&](const tpk::BuildDev& b, uint64_t rows) -> tp_status {
         mark_launch(e);
-        TP_TRY_CUDA(tpk::launch_build_part(b, rows, pj.counts, pj.cursor, (int64_t*)skeys, (uint32_t*)spays,
+        if (!pj.spill_mask) return cuda_check(tpk::launch_build(b, rows, e->num_sms, st), "build");
+        const uint64_t k = bi++;
+        TP_TRY_CUDA(tpk::launch_build_part(b, rows, bcounts + k * P, bcursor + k * P, (int64_t*)skeys, (uint32_t*)spays,
                                            e->num_sms, st));
-        for (int p = 0; p < P; ++p) {
-            if (!((pj.spill_mask >> p) & 1ull) || bc[p] == 0) continue;
+        for (int p = 0; p < P; ++p) {   // the next batch's scatter follows these copies on the stream
+            const uint64_t n = bc[k * P + p], at = base[k * P + p];
+            if (!((pj.spill_mask >> p) & 1ull) || n == 0) continue;
             tp_status r = append_device_rows(e, pj.build_spill[p],
-                                             {(const int64_t*)skeys + base[p], (const uint32_t*)spays + base[p]}, bc[p],
-                                             st);
+                                             {(const int64_t*)skeys + at, (const uint32_t*)spays + at}, n, st, false);
             if (r) return r;
         }
         return TP_OK;
     });
+    return s;   // phase 2 reads the pages on the same stream, after these copies
 }
 
 // Copies every partition's accumulated rows of the current set to its spill
@@ -1339,6 +1357,22 @@ tp_status part_acc_setup(ExecState& S, Scratch& sc, PartJoin& pj) {
     return TP_OK;
 }
 
+// Counts a fact batch's rows per spilled partition.  Called before the batch's
+// aggregate is launched, which then covers the counts' way to the host, where
+// part_spill_fact sizes the scatter by them.
+tp_status part_count_fact(ExecState& S, PartJoin& pj, const tpk::QueryDev& q, uint64_t rows) {
+    if (!pj.spill_mask || !pj.spill_fact || rows == 0) return TP_OK;
+    cudaStream_t st = S.lane->compute;
+    const uint64_t bytes = 8 * (uint64_t)pj.P;
+    if (!pj.counted) TP_TRY_CUDA(cudaEventCreateWithFlags(&pj.counted, cudaEventDisableTiming));
+    TP_TRY_CUDA(cudaMemsetAsync(pj.counts, 0, 2 * bytes, st));
+    mark_launch(S.e);
+    TP_TRY_CUDA(tpk::launch_part_hist_fact(q, rows, pj.shift, pj.spill_mask, pj.counts, S.e->num_sms, st));
+    TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words + PART_WORDS, pj.counts, bytes, cudaMemcpyDeviceToHost, st));
+    TP_TRY_CUDA(cudaEventRecord(pj.counted, st));
+    return TP_OK;
+}
+
 // Fact rows of spilled partitions in this batch go to their spill tables.
 tp_status part_spill_fact(ExecState& S, Scratch& sc, PartJoin& pj, const tpk::QueryDev& q, uint64_t rows,
                           const std::vector<const void*>& colptr) {
@@ -1346,12 +1380,9 @@ tp_status part_spill_fact(ExecState& S, Scratch& sc, PartJoin& pj, const tpk::Qu
     tp_engine* e = S.e;
     cudaStream_t st = S.lane->compute;
     const int P = pj.P;
-    TP_TRY_CUDA(cudaMemsetAsync(pj.counts, 0, 2 * 8 * (uint64_t)P, st));
-    mark_launch(e);
-    TP_TRY_CUDA(tpk::launch_part_hist_fact(q, rows, pj.shift, pj.spill_mask, pj.counts, e->num_sms, st));
-    std::vector<unsigned long long> bc(P), base(P, 0);
-    TP_TRY_CUDA(cudaMemcpyAsync(bc.data(), pj.counts, 8 * (uint64_t)P, cudaMemcpyDeviceToHost, st));
-    TP_TRY_CUDA(cudaStreamSynchronize(st));
+    TP_TRY_CUDA(cudaEventSynchronize(pj.counted));
+    const uint64_t* counted = S.lane->host_words + PART_WORDS;
+    std::vector<unsigned long long> bc(counted, counted + P), base(P, 0);
     uint64_t total = 0;
     for (int p = 0; p < P; ++p) {
         base[p] = total;
@@ -2073,7 +2104,8 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             }), "aggregate");
         };
         auto shared_batch = [&](const tpk::QueryDev& q, uint64_t rows, const std::vector<const void*>& colptr) {
-            tp_status r = shared_core(q, rows);
+            tp_status r = pj.on ? part_count_fact(S, pj, q, rows) : TP_OK;
+            if (r == TP_OK) r = shared_core(q, rows);
             if (r == TP_OK && pj.on) r = part_spill_fact(S, sc, pj, q, rows, colptr);
             return r;
         };
@@ -2291,7 +2323,8 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
                 }), "aggregate");
             };
             auto global_batch = [&](const tpk::QueryDev& q, uint64_t rows, const std::vector<const void*>& colptr) {
-                tp_status r = global_core(q, rows);
+                tp_status r = pj.on ? part_count_fact(S, pj, q, rows) : TP_OK;
+                if (r == TP_OK) r = global_core(q, rows);
                 if (r == TP_OK && pj.on) r = part_spill_fact(S, sc, pj, q, rows, colptr);
                 return r;
             };
