@@ -230,37 +230,64 @@ __global__ void __launch_bounds__(REC_THREADS, NS > 2 ? 2 : 4)
     }
 }
 
+// 32-bit atomics and loads at shared-memory addresses: through generic pointers
+// the hashed partitions took 400 us for 30M records, this way 336.
+__device__ __forceinline__ uint32_t sm_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void sm_red(uint32_t a, uint32_t v) {
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t sm_add(uint32_t a, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
+    return old;
+}
+__device__ __forceinline__ uint32_t sm_cas(uint32_t a, uint32_t was, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(old) : "r"(a), "r"(was), "r"(v) : "memory");
+    return old;
+}
+__device__ __forceinline__ uint32_t sm_ld(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
 // Adds a record's count and sums to slot k of a table of K slots in shared
-// memory: count[K], then low[K], high[K] per sum.
+// memory at cnt: count[K], then low[K], high[K] per sum.
 template <int NS>
-__device__ __forceinline__ void add_record(uint32_t* cnt, uint32_t K, uint32_t k, int n_sum, uint32_t c,
+__device__ __forceinline__ void add_record(uint32_t cnt, uint32_t K, uint32_t k, int n_sum, uint32_t c,
                                            const uint64_t v[NS]) {
-    atomicAdd(cnt + k, c);
+    uint32_t a = cnt + 4 * k;
+    sm_red(a, c);
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
         if (s >= n_sum) break;
-        uint32_t* lo = cnt + (uint64_t)K * (1 + 2 * s) + k;
-        const uint32_t old = atomicAdd(lo, (uint32_t)v[s]);
+        a += 4 * K;
+        const uint32_t old = sm_add(a, (uint32_t)v[s]);
+        a += 4 * K;
         const uint32_t h = (uint32_t)(v[s] >> 32) + (old + (uint32_t)v[s] < old ? 1u : 0u);
-        if (h) atomicAdd(lo + K, h);
+        if (h) sm_red(a, h);
     }
 }
 
-// Calls fn(key, rows, sums) for every record of partition p, each way's list
-// by the threads of its own share of the CTA, RAGG_UNROLL records' loads per
-// thread ahead of their use.
+// Calls fn(on, key, rows, sums) for every record of partition p (on: this lane
+// has one; all lanes of a warp make the same calls), each way's list by the
+// warps of its own share of the CTA, RAGG_UNROLL records' loads per thread
+// ahead of their use.
 constexpr int RAGG_UNROLL = 4;
 template <int NS, class F>
 __device__ __forceinline__ void for_each_record(const RecDev& rec, uint32_t p, int n_sum, F&& fn) {
     constexpr uint32_t SHARE = RAGG_THREADS / REC_WAYS;
+    static_assert(SHARE % 32 == 0, "a warp reads one list");
     const uint32_t list = p * REC_WAYS + threadIdx.x / SHARE;
     const uint32_t n = min(rec.cursor[(uint64_t)list * REC_CURSOR_STRIDE], rec.cap);
-    for (uint32_t i0 = threadIdx.x % SHARE; i0 < n; i0 += SHARE * RAGG_UNROLL) {
+    for (uint32_t i0 = 0; i0 < n; i0 += SHARE * RAGG_UNROLL) {
         uint4 r[RAGG_UNROLL];
         uint64_t v[RAGG_UNROLL][NS];
 #pragma unroll
         for (int u = 0; u < RAGG_UNROLL; ++u) {
-            const uint32_t i = i0 + u * SHARE;
+            const uint32_t i = i0 + u * SHARE + threadIdx.x % SHARE;
+            r[u] = make_uint4(0, 0, 0, 0);
             if (i >= n) continue;
             const uint64_t w = rec_at(rec, list, i);
             r[u] = __ldcs(rec.r0 + w);
@@ -270,9 +297,8 @@ __device__ __forceinline__ void for_each_record(const RecDev& rec, uint32_t p, i
         }
 #pragma unroll
         for (int u = 0; u < RAGG_UNROLL; ++u) {
-            if (i0 + u * SHARE >= n) break;
             v[u][0] = (uint64_t)r[u].w << 32 | r[u].z;
-            if (!fn(r[u].x, r[u].y, v[u])) return;
+            fn(i0 + u * SHARE + threadIdx.x % SHARE < n, r[u].x, r[u].y, v[u]);
         }
     }
 }
@@ -293,9 +319,8 @@ __global__ void __launch_bounds__(RAGG_THREADS)
     for (uint32_t i = threadIdx.x; i < words; i += RAGG_THREADS) rsm[i] = 0;
     __syncthreads();
     for (uint32_t p = blockIdx.x; p < rec.n_part; p += gridDim.x) {
-        for_each_record<NS>(rec, p, n_sum, [&](uint32_t k, uint32_t c, const uint64_t (&v)[NS]) {
-            add_record<NS>(rsm, K, k, n_sum, c, v);
-            return true;
+        for_each_record<NS>(rec, p, n_sum, [&](bool on, uint32_t k, uint32_t c, const uint64_t (&v)[NS]) {
+            if (on) add_record<NS>(sm_addr(rsm), K, k, n_sum, c, v);
         });
         __syncthreads();   // every record is read: the groups go over them
         const uint32_t kb = min(warp * per, K), ke = min(kb + per, K);
@@ -359,27 +384,36 @@ __global__ void __launch_bounds__(RAGG_THREADS)
         for (uint32_t i = threadIdx.x; i < REC_HASH; i += RAGG_THREADS) keys[i] = REC_NO_KEY;
         for (uint32_t i = threadIdx.x; i <= REC_ORDER; i += RAGG_THREADS) first[i] = 0;
         __syncthreads();
-        for_each_record<NS>(rec, p, n_sum, [&](uint32_t key, uint32_t c, const uint64_t (&v)[NS]) {
-            // most records meet a key that is there: find it with plain
-            // loads, claim only at an empty slot
-            uint32_t s = (key * 0x9E3779B1u) >> (32 - REC_HASH_BITS), left = REC_HASH;
-            for (;;) {
-                uint32_t k = ((volatile uint32_t*)keys)[s];
-                if (k == key) break;
+        // most records meet a key that is there: find it with plain loads, claim
+        // only at an empty slot.  The walk goes on for the whole warp until its
+        // last lane is done: left to themselves the lanes came out of it one by
+        // one and did the rest apart (8 of 32 lanes busy on average, 336 us for
+        // 30M records; 290 now, 20 lanes).
+        for_each_record<NS>(rec, p, n_sum, [&](bool on, uint32_t key, uint32_t c, const uint64_t (&v)[NS]) {
+            uint32_t s = (key * 0x9E3779B1u) >> (32 - REC_HASH_BITS), left = on ? REC_HASH : 0;
+            while (__any_sync(0xffffffffu, left != 0)) {
+                if (left == 0) continue;
+                uint32_t k = sm_ld(sm_addr(keys) + 4 * s);
                 if (k == REC_NO_KEY) {
-                    k = atomicCAS(keys + s, REC_NO_KEY, key);
-                    if (k == REC_NO_KEY) atomicAdd(first + 1 + (key >> bshift), 1u);
-                    if (k == REC_NO_KEY || k == key) break;
+                    k = sm_cas(sm_addr(keys) + 4 * s, REC_NO_KEY, key);
+                    if (k == REC_NO_KEY) {
+                        sm_red(sm_addr(first + 1) + 4 * (key >> bshift), 1u);
+                        k = key;
+                    }
+                }
+                if (k == key) {
+                    left = 0;
+                    continue;
                 }
                 s = (s + 1) & (REC_HASH - 1u);
                 // a full table; one that is full in another partition means this one need not go on
                 if (--left == 0 || ((left & 127u) == 0 && (*(volatile uint32_t*)err & ERR_RECORDS))) {
                     atomicOr(err, ERR_RECORDS);
-                    return false;
+                    left = 0;
+                    on = false;
                 }
             }
-            add_record<NS>(cnt, REC_HASH, s, n_sum, c, v);
-            return true;
+            if (on) add_record<NS>(sm_addr(cnt), REC_HASH, s, n_sum, c, v);
         });
         __syncthreads();
         // bucket starts: an inclusive scan of first[1 ..]
