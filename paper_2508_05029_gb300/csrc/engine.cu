@@ -75,8 +75,25 @@ tp_status dev_alloc(tp_engine* e, void** p, uint64_t bytes, cudaStream_t st) {
     return TP_OK;
 }
 
+// A batch's column in its pages when its extents follow one another in memory,
+// nullptr otherwise.
+static const uint8_t* page_column(tp_engine* e, const Batch& b, int c) {
+    const uint8_t *first = nullptr, *end = nullptr;
+    for (const Extent& x : b.cols[c]) {
+        const uint8_t* p = (const uint8_t*)tp_page_ptr(e, x.page) + x.offset;
+        if (!first) first = p;
+        else if (p != end) return nullptr;
+        end = p + x.bytes;
+    }
+    return first;
+}
+
 tp_status copy_batch_column(tp_engine* e, const tp_table* t, const Batch& b, int c, void* full, void* enc,
-                            uint64_t row_off, cudaStream_t st, uint8_t** stage) {
+                            uint64_t row_off, cudaStream_t st, uint8_t** stage, bool in_place) {
+    if (in_place && b.narrow(c) && page_column(e, b, c)) {   // widened straight from its pages
+        e->h2d_bytes += b.packed(c) ? (b.rows * b.enc_bits[c] + 7) / 8 : b.stored_bytes(c, t->types[c]);
+        return TP_OK;
+    }
     // a narrow column's rows land at its widest encoding's offsets (enc holds
     // narrow_width_max bytes per row)
     const uint64_t sz = b.narrow(c) ? (uint64_t)narrow_width_max(t, c) : type_size(t->types[c]);
@@ -109,6 +126,7 @@ namespace {
 struct Widener {
     tp_engine* e;
     cudaStream_t st;
+    bool in_place;
     tpk::DecodeCols d{};
     tp_status flush() {
         if (d.n == 0) return TP_OK;
@@ -135,14 +153,15 @@ struct Widener {
             }
             const uint64_t sz = type_size(t->types[c]);
             const uint64_t wmax = (uint64_t)narrow_width_max(t, c);
-            const uint8_t* src = (const uint8_t*)enc[i] + row_off * wmax;
+            const uint8_t* pages = in_place ? page_column(e, b, c) : nullptr;
+            const uint8_t* src = pages ? pages : (const uint8_t*)enc[i] + row_off * wmax;
             const int k = last[i];
-            if (k >= 0 && !b.packed(c) && d.bits[k] == 0 && d.w[k] == b.enc_w[c] && b.enc_w[c] == wmax &&
+            if (k >= 0 && !pages && !b.packed(c) && d.bits[k] == 0 && d.w[k] == b.enc_w[c] && b.enc_w[c] == wmax &&
                 d.base[k] == b.enc_base[c] && (const uint8_t*)d.src[k] + d.rows[k] * wmax == src) {
                 d.rows[k] += b.rows;
                 continue;
             }
-            last[i] = d.n;
+            last[i] = pages ? -1 : d.n;
             d.src[d.n] = src;
             d.dst[d.n] = (uint8_t*)full[i] + row_off * sz;
             d.base[d.n] = b.enc_base[c];
@@ -164,14 +183,15 @@ struct Widener {
 tp_status widen_batch(tp_engine* e, const tp_table* t, const Batch& b, const std::vector<int>& cols,
                       const std::vector<void*>& full, const std::vector<void*>& enc, uint64_t row_off,
                       cudaStream_t st) {
-    Widener w{e, st};
+    Widener w{e, st, false};
     tp_status s = w.add(t, b, cols, full, enc, row_off);
     return s ? s : w.flush();
 }
 
 tp_status widen_batches(tp_engine* e, const tp_table* t, size_t first, size_t last, const std::vector<int>& cols,
-                        const std::vector<void*>& full, const std::vector<void*>& enc, cudaStream_t st) {
-    Widener w{e, st};
+                        const std::vector<void*>& full, const std::vector<void*>& enc, cudaStream_t st,
+                        bool in_place) {
+    Widener w{e, st, in_place};
     uint64_t row_off = 0;
     for (size_t bi = first; bi < last; ++bi) {
         tp_status s = w.add(t, t->batches[bi], cols, full, enc, row_off);

@@ -285,9 +285,11 @@ std::string geometry_macros(const tpk::StageGeom& geom);
 // full-width column lands at full + row_off * size, a narrow one at
 // enc + row_off * size (enc is then widened by widen_batch).  Adds the bytes
 // to the engine's counter.  With stage, the bytes are first copied on the
-// host to *stage (page-locked, advanced past them) and sent from there.
+// host to *stage (page-locked, advanced past them) and sent from there.  With
+// in_place, a narrow column that lies in one piece in its pages is not copied:
+// the widening (in_place there too) reads it over the link.
 tp_status copy_batch_column(tp_engine* e, const tp_table* t, const Batch& b, int c, void* full, void* enc,
-                            uint64_t row_off, cudaStream_t st, uint8_t** stage = nullptr);
+                            uint64_t row_off, cudaStream_t st, uint8_t** stage = nullptr, bool in_place = false);
 // Widens batch b's narrow columns among cols (enc -> full, the offsets of
 // copy_batch_column at row_off) with one launch on st.
 tp_status widen_batch(tp_engine* e, const tp_table* t, const Batch& b, const std::vector<int>& cols,
@@ -297,7 +299,8 @@ tp_status widen_batch(tp_engine* e, const tp_table* t, const Batch& b, const std
 // same slots (each at the rows of the ones before it), in as few launches as
 // the decode descriptor allows.
 tp_status widen_batches(tp_engine* e, const tp_table* t, size_t first, size_t last, const std::vector<int>& cols,
-                        const std::vector<void*>& full, const std::vector<void*>& enc, cudaStream_t st);
+                        const std::vector<void*>& full, const std::vector<void*>& enc, cudaStream_t st,
+                        bool in_place = false);
 // Narrowest frame-of-reference width (1, 2 or 4 bytes) for values in [lo,
 // hi] of a column of full width `full`, or 0 when it saves nothing.
 int frame_width(int64_t lo, int64_t hi, int full);
