@@ -957,9 +957,22 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     at += cnt_bytes;
     unsigned long long* offsets = (unsigned long long*)at;
     TP_TRY_CUDA(cudaMemsetAsync(rec.cursor, 0, cur_bytes, st));
-    // ---- records
+    // ---- records, by the scan compiled for the plan's shape where that is to be had
     e->batches++;
-    if (sel && tpk::select_usable(q, std::min(rows, sel_rows))) {
+    const bool selected = sel && tpk::select_usable(q, std::min(rows, sel_rows));
+    const void* jk = nullptr;
+    if (!(e->cfg.flags & TP_FLAG_NO_JIT)) {
+        std::string why;
+        const int8_t modes[tpk::MAX_SUM] = {};
+        const int narrow[tpk::MAX_SUM] = {};
+        jk = plan_kernel(p, q, modes, selected ? -2 : -1, narrow, tpk::JIT_RECORDS_GEOM, [&] {
+            return jit_kernel(e, geometry_macros(tpk::JIT_RECORDS_GEOM) +
+                                     (selected ? "#define TPJ_SELECTED 1\n" : "") +
+                                     shape_struct("JS", q, modes, false, true, narrow) +
+                                     "#include \"jit_records.cuh\"\n", "tpj_records", &why);
+        });
+    }
+    if (selected) {
         for (uint64_t off = 0; off < rows; off += sel_rows) {
             const uint64_t nr = std::min(sel_rows, rows - off);
             const tpk::QueryDev qs = off ? tpk::offset_rows(q, off) : q;
@@ -969,26 +982,17 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
             s = cuda_check(timer.run(st, nr, [&] {
                 cudaError_t ce = tpk::launch_select(qs, nr, sel, sel_cursor, e->num_sms, st);
                 if (ce != cudaSuccess) return ce;
-                return tpk::launch_rec_selected(qs, sel, sel_cursor, nr, rec, e->num_sms, st);
+                return jk ? tpk::launch_rec_scan_jit(jk, qs, nr, sel, sel_cursor, rec, e->num_sms, st)
+                          : tpk::launch_rec_selected(qs, sel, sel_cursor, nr, rec, e->num_sms, st);
             }), "aggregate");
             if (s) return s;
+            if (jk) e->jit_launches++;
         }
     } else {
         mark_launch(e);
-        const void* jk = nullptr;
-        if (!(e->cfg.flags & TP_FLAG_NO_JIT)) {
-            std::string why;
-            const int8_t modes[tpk::MAX_SUM] = {};
-            const int narrow[tpk::MAX_SUM] = {};
-            jk = plan_kernel(p, q, modes, -1, narrow, tpk::JIT_RECORDS_GEOM, [&] {
-                return jit_kernel(e, geometry_macros(tpk::JIT_RECORDS_GEOM) +
-                                         shape_struct("JS", q, modes, false, true, narrow) +
-                                         "#include \"jit_records.cuh\"\n", "tpj_records", &why);
-            });
-            if (jk) e->jit_launches++;
-        }
+        if (jk) e->jit_launches++;
         s = cuda_check(timer.run(st, rows, [&] {
-            return jk ? tpk::launch_rec_scan_jit(jk, q, rows, rec, e->num_sms, st)
+            return jk ? tpk::launch_rec_scan_jit(jk, q, rows, nullptr, nullptr, rec, e->num_sms, st)
                       : tpk::launch_rec_scan(q, rows, rec, e->num_sms, st);
         }), "aggregate");
         if (s) return s;

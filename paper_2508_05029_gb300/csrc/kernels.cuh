@@ -462,9 +462,10 @@ cudaError_t launch_agg_selected(const QueryDev& q, const uint32_t* sel, const un
 // Group fields all in the fact table, no further joins, no fan-out, n_sum <=
 // REC_MAX_SUM, fewer than 2^32 rows, 16-byte aligned columns.
 cudaError_t launch_rec_scan(const QueryDev& q, uint64_t n, const RecDev& rec, int num_sms, cudaStream_t st);
-// The same launch of a run-time compiled scan (tpj_records).
-cudaError_t launch_rec_scan_jit(const void* kernel, const QueryDev& q, uint64_t n, const RecDev& rec, int num_sms,
-                                cudaStream_t st);
+// The same launch of a run-time compiled scan (tpj_records): of all n rows, or
+// with sel of the *count selected ones (at most n).
+cudaError_t launch_rec_scan_jit(const void* kernel, const QueryDev& q, uint64_t n, const uint32_t* sel,
+                                const unsigned long long* count, const RecDev& rec, int num_sms, cudaStream_t st);
 // The *count rows of a selection vector (launch_select), at most max_rows.
 cudaError_t launch_rec_selected(const QueryDev& q, const uint32_t* sel, const unsigned long long* count,
                                 uint64_t max_rows, const RecDev& rec, int num_sms, cudaStream_t st);

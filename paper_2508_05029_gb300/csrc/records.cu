@@ -609,8 +609,8 @@ cudaError_t launch_rec_scan(const QueryDev& q, uint64_t n, const RecDev& rec, in
     return rec_scan_t<REC_MAX_SUM>(q, n, rec, num_sms, st);
 }
 
-cudaError_t launch_rec_scan_jit(const void* kernel, const QueryDev& q, uint64_t n, const RecDev& rec, int num_sms,
-                                cudaStream_t st) {
+cudaError_t launch_rec_scan_jit(const void* kernel, const QueryDev& q, uint64_t n, const uint32_t* sel,
+                                const unsigned long long* count, const RecDev& rec, int num_sms, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, REC_THREADS, 0);
@@ -619,7 +619,7 @@ cudaError_t launch_rec_scan_jit(const void* kernel, const QueryDev& q, uint64_t 
     const unsigned grid = (unsigned)std::min<uint64_t>(blocks, (uint64_t)num_sms * std::max(per_sm, 1));
     QueryDev qa = q;
     RecDev ra = rec;
-    void* args[] = {&qa, &n, &ra};
+    void* args[] = {&qa, &n, &sel, &count, &ra};
     return cudaLaunchKernel(kernel, dim3(grid), dim3(REC_THREADS), args, 0, st);
 }
 

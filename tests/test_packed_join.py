@@ -96,13 +96,14 @@ def test_errors_of_a_packed_join(built, flags):
         e.close()
 
 
+@pytest.mark.parametrize("selected", ["", "#define TPJ_SELECTED 1\n"])
 @pytest.mark.parametrize("shape", [
     _shape(groups=((0, 1, 64),), sums=((1, 1, 1, 0, 0),), fast=False),
     _shape(join=4, ktype=1, groups=((0, 0, 10), (0, 1, 10)), fast=False,
            sums=((0, 1, 0, 0, 0), (0, 2, 0, 0, 0), (1, 1, 0, 0, 0), (0, 0, 0, 0, 0))),
     _shape(join=0, filter=0, groups=((0, 1, 64),), sums=(), fast=False)])
-def test_nvrtc_compiles_record_scans(shape, monkeypatch):
+def test_nvrtc_compiles_record_scans(shape, selected, monkeypatch):
     from tests import test_jit_source
     monkeypatch.setattr(test_jit_source, "HEADERS", test_jit_source.HEADERS + ["records.cuh", "jit_records.cuh"])
     _compile(_nvrtc(), "#undef TP_ST_CONSUMERS\n#undef TP_ST_RPL\n#define TP_ST_CONSUMERS 8\n#define TP_ST_RPL 4\n" +
-             shape + '#include "jit_records.cuh"\n')
+             selected + shape + '#include "jit_records.cuh"\n')
