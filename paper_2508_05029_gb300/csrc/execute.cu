@@ -127,15 +127,18 @@ struct Scratch {
         total = at = 0;
         uint64_t held = 0, cap = 0;
         if (want <= lane->arena_bytes || tp_budget_query(e, &held, &cap) != TP_OK) return;
-        if (e->arena_total - lane->arena_bytes + want > std::min(ARENA_MAX, cap / 8)) return;
+        if ((e->arena_total += want) - lane->arena_bytes > std::min(ARENA_MAX, cap / 8)) {
+            e->arena_total -= want;   // counted first: other lanes grow theirs at the same time
+            return;
+        }
         lane_drop_arena(e, lane);
         if (cudaMallocAsync(&lane->arena, want, st) != cudaSuccess) {
             cudaGetLastError();
             lane->arena = nullptr;
+            e->arena_total -= want;
             return;
         }
         lane->arena_bytes = want;
-        e->arena_total += want;
     }
     ~Scratch() { free_all(); }
 };
@@ -997,7 +1000,10 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
         }), "aggregate");
         if (s) return s;
     }
-    TP_TRY_CUDA(tpk::launch_rec_aggregate(rec, ns, hashed, n_groups, S.err, e->num_sms, st));
+    s = cuda_check(timer.run(st, 0, [&] {
+        return tpk::launch_rec_aggregate(rec, ns, hashed, n_groups, S.err, e->num_sms, st);
+    }), "aggregate");
+    if (s) return s;
     TP_TRY_CUDA(tpk::launch_direct_scan(n_groups, rec.n_part, offsets, st));
     mark_launch(e);
     mark_launch(e);

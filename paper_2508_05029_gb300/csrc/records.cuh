@@ -75,8 +75,8 @@ __device__ __forceinline__ void fold_append(const QueryDev& q, const RecDev& rec
     for (int i = 0; i < REC_RPT; ++i) {
         local[i] = key[i] - rec.kmin;
         cnt[i] = 1;
-        if (pass[i] && local[i] >= rec.span) {   // outside the column bounds: cannot happen
-            atomicOr(q.err, ERR_INTERNAL);
+        if (pass[i] && local[i] >= rec.span) {   // a caller's column changed since its bounds were taken
+            atomicOr(q.err, ERR_RECORDS);
             pass[i] = false;
         }
     }
