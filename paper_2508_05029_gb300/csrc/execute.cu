@@ -816,9 +816,9 @@ const void* plan_kernel(tp_plan* p, const tpk::QueryDev& q, const int8_t* mode, 
 // Records (records.cu) pay when the global table they replace would be
 // updated out of L2: from REC_MIN_ROWS fact rows, and groups or a key range
 // that make its table REC_MIN_GROUPS slots or more.  At 60M rows, 15M groups
-// next to each other in the rows: 0.79 ms per query against 1.38 ms through
-// the direct-addressed table; 30M rows, 3M sparse groups in no order: 1.00
-// against 1.48 ms; 600k groups selected from 60M rows: 0.24 against 0.35 ms.
+// next to each other in the rows: 0.78 ms per query against 1.38 ms through
+// the direct-addressed table; 30M rows, 3M sparse groups in no order: 0.86
+// against 1.48 ms; 600k groups selected from 60M rows: 0.22 against 0.35 ms.
 constexpr uint64_t REC_MIN_ROWS = 4ull << 20;
 constexpr uint64_t REC_MIN_GROUPS = 1ull << 18;
 constexpr uint32_t REC_SAMPLES = 1u << 16;
