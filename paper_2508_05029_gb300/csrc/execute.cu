@@ -348,19 +348,25 @@ tp_status build_join_many(ExecState& S, Scratch& sc) {
     });
     if (s) return s;
     unsigned long long* total = (unsigned long long*)ctr;
-    TP_TRY_CUDA(tpk::launch_many_starts(S.jt, (uint2*)rows_out, total, e->num_sms, st));
+    uint32_t fan = S.p->fan;
+    TP_TRY_CUDA(tpk::launch_many_starts(S.jt, (uint2*)rows_out, total, fan ? fan : ~0u, S.err, e->num_sms, st));
     mark_launch(e);
-    if (n_rows >= (1ull << 31)) {   // only then can too many rows be admitted
-        TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words, total, 8, cudaMemcpyDeviceToHost, st));
+    // only from 2^31 rows on can too many be admitted; the longest run is read
+    // here once per plan, later executions only check it
+    if (n_rows >= (1ull << 31) || fan == 0) {
+        TP_TRY_CUDA(cudaMemcpyAsync(S.lane->host_words, total, 16, cudaMemcpyDeviceToHost, st));
         TP_TRY_CUDA(cudaStreamSynchronize(st));
+        e->d2h_bytes += 16;
         if (S.lane->host_words[0] >= (1ull << 31))
             return fail(TP_E_INVALID, "fan-out join: more than 2^31 build rows");
+        if (fan == 0) S.p->fan = fan = (uint32_t)std::max<uint64_t>(1, S.lane->host_words[1]);
     }
     TP_TRY_CUDA(tpk::launch_many_place(S.jt, (uint32_t*)pays, (uint64_t*)place, n_rows, (uint2*)rows_out, e->num_sms,
                                        st));
     mark_launch(e);
     S.jt.mrow = (uint2*)rows_out;
     S.jt.many = 1;
+    S.jt.fan = fan;
     return TP_OK;
 }
 
@@ -587,8 +593,12 @@ tp_status sample_dim_selectivity(ExecState& S, int k) {
 // Internal status: a packed join table could not hold its rows; the query runs
 // again with unpacked ones.
 constexpr tp_status RETRY_UNPACKED = -1;
+// Internal status: a fan-out key has more build rows than the plan's bound; the
+// query runs again with the rows counted first.
+constexpr tp_status RETRY_FANOUT = -3;
 
 tp_status map_err(uint32_t err) {
+    if (err & tpk::ERR_FANOUT) return RETRY_FANOUT;
     if (err & tpk::ERR_PACKED) return RETRY_UNPACKED;
     if (err & tpk::ERR_DUP) return fail(TP_E_DUP_KEY, "join build side holds a duplicate key");
     if (err & tpk::ERR_RANGE) return fail(TP_E_RANGE, "a group field value does not fit its bit width");
@@ -2049,7 +2059,8 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             return plain_grid;
         };
         const bool want_staged = !(e->cfg.flags & TP_FLAG_NO_STAGED);
-        bool fast = want_staged && !(e->cfg.flags & TP_FLAG_EXACT_ONLY) && sums_fit_int64(p, S.fact);
+        const uint64_t fan = S.jt.many ? S.jt.fan : 1;
+        bool fast = want_staged && !(e->cfg.flags & TP_FLAG_EXACT_ONLY) && sums_fit_int64(p, S.fact, fan);
         tpk::TermBounds bounds[tpk::MAX_SUM] = {};
         if (want_staged) term_bounds(p, S.fact, bounds);
         int narrow[tpk::MAX_SUM] = {};
@@ -2077,9 +2088,9 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
                     // sums that may leave int64 as 32-bit limbs: 64-bit shared
                     // atomics only where the limbs' rows do not fit (or on request)
                     tpk::StageLayout LJ;
-                    const tpk::DenseWords dw = mode == 2                                 ? tpk::DW_FAST
-                                               : (e->cfg.flags & TP_FLAG_EXACT_ONLY) != 0 ? tpk::DW_EXACT
-                                                                                          : tpk::DW_WIDE;
+                    tpk::DenseWords dw = mode == 2                                 ? tpk::DW_FAST
+                                         : (e->cfg.flags & TP_FLAG_EXACT_ONLY) != 0 ? tpk::DW_EXACT
+                                                                                    : tpk::DW_WIDE;
                     bool hashed = q.has_join && !q.jt.direct;
                     for (int j = 0; j < q.n_xjoin; ++j) hashed = hashed || !q.jtx[j].direct;
                     auto layout = [&](const tpk::StageGeom& geom, int stages) {
@@ -2087,12 +2098,17 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
                                                          &LJ) &&
                                rows >= (uint64_t)LJ.tile;
                     };
-                    const tpk::StageGeom* geom = nullptr;
-                    if (!hashed && layout(tpk::JIT_DENSE_GEOM, tpk::JIT_DENSE_STAGES) &&
-                        LJ.n_stages == tpk::JIT_DENSE_STAGES)
-                        geom = &tpk::JIT_DENSE_GEOM;
-                    else if (layout(tpk::JIT_HASHED_GEOM, tpk::JIT_HASHED_STAGES))
-                        geom = &tpk::JIT_HASHED_GEOM;
+                    auto pick = [&]() -> const tpk::StageGeom* {
+                        if (!hashed && layout(tpk::JIT_DENSE_GEOM, tpk::JIT_DENSE_STAGES) &&
+                            LJ.n_stages == tpk::JIT_DENSE_STAGES)
+                            return &tpk::JIT_DENSE_GEOM;
+                        return layout(tpk::JIT_HASHED_GEOM, tpk::JIT_HASHED_STAGES) ? &tpk::JIT_HASHED_GEOM : nullptr;
+                    };
+                    const tpk::StageGeom* geom = pick();
+                    if (!geom && dw != tpk::DW_EXACT && q.jt.many) {   // partners beyond 32-bit words
+                        dw = tpk::DW_EXACT;
+                        geom = pick();
+                    }
                     if (geom) {
                         std::string why;
                         jk = plan_kernel(S.p, q, LJ.sum_mode, dw, narrow, *geom, [&] {
@@ -2166,7 +2182,8 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
         // staged); 64-bit low-word updates when column bounds rule out
         // overflow (any mix of the kernels then agrees on the low words)
         const bool g_staged = !(e->cfg.flags & TP_FLAG_NO_STAGED);
-        const bool gfast = g_staged && !(e->cfg.flags & TP_FLAG_EXACT_ONLY) && sums_fit_int64(p, S.fact);
+        const bool gfast = g_staged && !(e->cfg.flags & TP_FLAG_EXACT_ONLY) &&
+                           sums_fit_int64(p, S.fact, S.jt.many ? S.jt.fan : 1);
         const bool stage_all = p->selectivity >= 0.25;
         uint32_t* sel = nullptr;
         unsigned long long* sel_cursor = (unsigned long long*)((uint8_t*)misc + 1024);
@@ -2452,13 +2469,13 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
 }
 
 tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out) {
-    tp_status s = execute_once(p, lane, cache, out);
-    if (s == RETRY_UNPACKED) {   // Section 3.3.2: a task retried with a better estimate
-        p->no_packed = true;
+    for (;;) {   // Section 3.3.2: a task retried with a better estimate
+        const tp_status s = execute_once(p, lane, cache, out);
+        if (s == RETRY_UNPACKED) p->no_packed = true;   // neither comes back once its estimate is dropped
+        else if (s == RETRY_FANOUT) p->fan = 0;
+        else return s;
         p->eng->retries++;
-        s = execute_once(p, lane, cache, out);
     }
-    return s;
 }
 
 }  // namespace
@@ -2516,7 +2533,7 @@ tpk::QueryDev plan_query_dev(const tp_plan* p, const std::vector<const void*>& c
 }
 
 // True when column bounds prove that every sum of the query stays inside
-// int64 over all n fact rows, so kernels may accumulate 64-bit values without
+// int64 over all n fact rows (a fan-out row counts once per partner), so kernels may accumulate 64-bit values without
 // carry handling.  |a| <= A and |K - b| <= D give |term| <= A * D < 2^127.
 bool direct_join_range(const tp_table* dim, int col, uint64_t* range) {
     if (dim->rows == 0) return false;
@@ -2526,7 +2543,7 @@ bool direct_join_range(const tp_table* dim, int col, uint64_t* range) {
     return true;
 }
 
-bool sums_fit_int64(const tp_plan* p, const tp_table* fact) {
+bool sums_fit_int64(const tp_plan* p, const tp_table* fact, uint64_t fan) {
     const uint64_t n = fact->rows;
     if (n == 0) return true;
     if (n >= (1ull << 32)) return false;   // per-CTA 32-bit counts
@@ -2544,7 +2561,7 @@ bool sums_fit_int64(const tp_plan* p, const tp_table* fact) {
             if (D > limit) return false;
             B = A * D;
         }
-        if (B > limit / (i128)n) return false;
+        if (B > limit / ((i128)n * (i128)fan)) return false;
     }
     return true;
 }

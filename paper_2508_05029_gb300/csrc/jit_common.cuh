@@ -204,7 +204,7 @@ __device__ __forceinline__ void sums(const QueryDev& q, const Tab& t, const C& c
         } else if constexpr (S::fast && S::mode[I] >= 3) {
             // exact sums as 32-bit limbs: 32-bit shared-memory atomics are
             // native where 64-bit ones are compare-and-swap loops.  Three
-            // limbs hold (term - offset) < 2^64 of up to 2^32 rows (the low
+            // limbs hold (term - offset) < 2^64 of up to 2^32 terms (the low
             // 64 bits of a * (k - b) - off are exact); four hold any term
             // modulo 2^128.  A fan-out query of 20M rows x 3 partners with one
             // three-limb sum: 1.80 ms with 64-bit words, 1.34 ms with limbs.

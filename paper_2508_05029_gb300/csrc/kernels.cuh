@@ -39,6 +39,7 @@ enum : uint32_t {
     ERR_TIMEOUT = 16u,   // a bounded device wait expired
     ERR_PACKED = 32u,    // a packed join table could not place a key: rerun with unpacked tables
     ERR_RECORDS = 64u,   // a record partition or its table is full: aggregate through the global table
+    ERR_FANOUT = 128u,   // a fan-out key has more rows than the plan's bound: rerun with its rows counted
 };
 
 constexpr uint64_t EMPTY64 = ~0ull;
@@ -101,7 +102,7 @@ struct JoinTable {
     // rows of the run follow it
     const uint2* mrow;
     int32_t many;
-    int32_t pad4;
+    uint32_t fan;           // no run is longer (partners of one fact row)
 };
 
 constexpr uint32_t PACK_DIST_BITS = 5;                            // at least this many distance bits
@@ -497,14 +498,15 @@ cudaError_t launch_part_hist(const BuildDev& b, uint64_t n, int shift, unsigned 
 // and writes every row's payload and place (table slot << MANY_RANK_BITS |
 // rank among the key's rows; MANY_NONE: not admitted), launch_many_starts
 // makes the slots' payloads the starts of their keys' runs and writes the runs'
-// lengths (*total: rows), and launch_many_place writes the rows into the runs.
+// lengths (total[0]: rows, total[1]: the longest run; one longer than limit:
+// ERR_FANOUT), and launch_many_place writes the rows into the runs.
 constexpr int MANY_RANK_BITS = 31;
 constexpr uint64_t MANY_NONE = ~0ull;
 constexpr uint64_t MANY_SIDE = (1ull << (64 - MANY_RANK_BITS)) - 2;   // the side cell's rows
 cudaError_t launch_many_count(const BuildDev& b, uint64_t n, uint32_t* pays, uint64_t* place, int num_sms,
                               cudaStream_t st);
-cudaError_t launch_many_starts(const JoinTable& jt, uint2* rows, unsigned long long* total, int num_sms,
-                               cudaStream_t st);
+cudaError_t launch_many_starts(const JoinTable& jt, uint2* rows, unsigned long long* total, uint32_t limit,
+                               uint32_t* err, int num_sms, cudaStream_t st);
 cudaError_t launch_many_place(const JoinTable& jt, const uint32_t* pays, const uint64_t* place, uint64_t n,
                               uint2* rows, int num_sms, cudaStream_t st);
 cudaError_t launch_part_hist_fact(const QueryDev& q, uint64_t n, int shift, uint64_t spill_mask,

@@ -350,19 +350,20 @@ cudaError_t launch_many_count(const BuildDev& b, uint64_t n, uint32_t* pays, uin
     return cudaGetLastError();
 }
 
-// Turns the counts of the table's slots into run starts; *total ends as the
-// number of rows.  One reservation on *total per tile of MS_TILE slots: one
-// per warp would queue on that word.
+// Turns the counts of the table's slots into run starts; total[0] ends as the
+// number of rows, total[1] as the longest run.  One reservation on *total per
+// tile of MS_TILE slots: one per warp would queue on that word.
 constexpr int MS_THREADS = 256;
 constexpr int MS_ITEMS = 16;
 constexpr int MS_TILE = MS_THREADS * MS_ITEMS;
 
 __global__ void __launch_bounds__(MS_THREADS)
     k_many_starts(const __grid_constant__ JoinTable jt, uint64_t n_slots, uint2* __restrict__ rows,
-                  unsigned long long* total) {
+                  unsigned long long* total, uint32_t limit, uint32_t* err) {
     __shared__ uint32_t warp_sum[MS_THREADS / 32];
     __shared__ unsigned long long base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t longest = 0;
     for (uint64_t t0 = (uint64_t)blockIdx.x * MS_TILE; t0 < n_slots; t0 += (uint64_t)gridDim.x * MS_TILE) {
         uint32_t cnt[MS_ITEMS], sum = 0;
 #pragma unroll
@@ -370,6 +371,7 @@ __global__ void __launch_bounds__(MS_THREADS)
             const uint64_t s = t0 + (uint64_t)j * MS_THREADS + threadIdx.x;
             cnt[j] = s < n_slots ? *many_word(jt, s) + 1u : 0u;
             sum += cnt[j];
+            longest = max(longest, cnt[j]);
         }
         uint32_t x = sum;
         for (int off = 1; off < 32; off <<= 1) {
@@ -402,15 +404,20 @@ __global__ void __launch_bounds__(MS_THREADS)
         const uint32_t n = jt.side[1], at = (uint32_t)atomicAdd(total, (unsigned long long)n);
         rows[at].y = n - 1u;
         jt.side[1] = at;
+        longest = max(longest, n);
     }
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    if (lane != 0 || longest == 0) return;
+    if (longest > limit) atomicOr(err, ERR_FANOUT);
+    atomicMax(total + 1, (unsigned long long)longest);
 }
 
-cudaError_t launch_many_starts(const JoinTable& jt, uint2* rows, unsigned long long* total, int num_sms,
-                               cudaStream_t st) {
+cudaError_t launch_many_starts(const JoinTable& jt, uint2* rows, unsigned long long* total, uint32_t limit,
+                               uint32_t* err, int num_sms, cudaStream_t st) {
     const uint64_t n_slots = jt.direct ? jt.range : jt.mask + 1;
     uint64_t blocks = (n_slots + MS_TILE - 1) / MS_TILE;
     if (blocks > (uint64_t)num_sms * 8) blocks = (uint64_t)num_sms * 8;
-    k_many_starts<<<(unsigned)blocks, MS_THREADS, 0, st>>>(jt, n_slots, rows, total);
+    k_many_starts<<<(unsigned)blocks, MS_THREADS, 0, st>>>(jt, n_slots, rows, total, limit, err);
     return cudaGetLastError();
 }
 

@@ -252,21 +252,23 @@ bool staged_layout_shared(const QueryDev& q, uint32_t key_bits, DenseWords kind,
         // rows one CTA can see in this launch bound every 32-bit word: its
         // share of the whole tiles plus, for the run-time compiled kernel, the
         // rows after the last whole tile, which CTA (tiles % grid) evaluates
-        // too -- CTA 0, holding a full share, when tiles is a multiple of grid
+        // too -- CTA 0, holding a full share, when tiles is a multiple of grid.
+        // Under fan-out a row adds its terms once per partner.
         const uint64_t tiles = rows / tile;
         const uint64_t grid = std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)num_sms * geom.ctas));
         const uint64_t r_cta = (tiles + grid - 1) / grid * (uint64_t)tile + (rows - tiles * (uint64_t)tile);
-        if (r_cta >= (1ull << 32)) return false;
+        const unsigned __int128 rs = (unsigned __int128)r_cta * (q.has_join && q.jt.many ? q.jt.fan : 1u);
+        if (rs >= (1ull << 32)) return false;
         uint32_t block = 1;   // block 0: counts
         for (int s = 0; s < q.n_sum; ++s) {
-            const unsigned __int128 rs = (unsigned __int128)r_cta, span = bounds[s].span;
+            const unsigned __int128 span = bounds[s].span;
             const bool off64 = bounds[s].lo >= INT64_MIN && bounds[s].lo <= INT64_MAX;
             if (off64 && span <= 0xFFFFFFFFull && rs * span <= 0xFFFFFFFFull) {
                 L->sum_mode[s] = 1;
             } else if (off64 && (span >> 64) == 0 && rs * ((span >> 32) + 1) <= 0xFFFFFFFFull) {
                 L->sum_mode[s] = 2;
             } else if (kind == DW_WIDE) {
-                // three limbs: fewer than 2^32 rows of terms below 2^64
+                // three limbs: fewer than 2^32 terms below 2^64
                 L->sum_mode[s] = off64 && (span >> 64) == 0 ? 3 : 4;
             } else {
                 return false;

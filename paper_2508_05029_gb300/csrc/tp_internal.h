@@ -187,6 +187,9 @@ struct tp_plan {
     // run-time compiled kernels by the bytes of their shape and geometry
     std::vector<std::pair<std::string, const void*>> kernels;
     bool no_packed = false;      // a packed join table could not place a key: unpacked ones from then on
+    // fan-out: most build rows of one key an execution met (0: none has counted
+    // them); the build of every execution checks it
+    uint32_t fan = 0;
 };
 
 struct tp_result {
@@ -262,8 +265,9 @@ bool direct_join_range(const tp_table* dim, int col, uint64_t* range);
 // negative or wider than its field).
 bool direct_group_range(const tp_plan* p, const tp_table* fact, const tp_table* dim, uint64_t* kmin,
                         uint64_t* span);
-// Column bounds prove every sum of the plan stays inside int64 over the fact table.
-bool sums_fit_int64(const tp_plan* p, const tp_table* fact);
+// Column bounds prove every sum of the plan stays inside int64 over the fact
+// table, each row adding its terms at most fan times.
+bool sums_fit_int64(const tp_plan* p, const tp_table* fact, uint64_t fan = 1);
 // Per-row term range of every sum slot.
 void term_bounds(const tp_plan* p, const tp_table* fact, tpk::TermBounds* out);
 // out[s] = 1 for MUL_SUB sum slots whose two factors fit in int32 by the
