@@ -543,6 +543,9 @@ tp_status tp_stats_get(tp_engine* eng, tp_stats* out);
 /* Fault injection for tests: the next n host page allocations and device
  * reservations fail as if exhausted. */
 tp_status tp_debug_fail_next_alloc(tp_engine* eng, int32_t n);
+/* The next n device allocations of at least min_bytes fail as if the device
+ * were out of memory. */
+tp_status tp_debug_fail_device_allocs(tp_engine* eng, uint64_t min_bytes, int32_t n);
 /* The page encoding of a bit-packed column, for tests (host only, no GPU):
  * packs values[0..n) (each below 2^bits, 1 <= bits <= 31) into
  * words[0..ceil(n * bits / 32)), value i at bits [i * bits, (i + 1) * bits)

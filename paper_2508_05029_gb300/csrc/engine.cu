@@ -37,6 +37,91 @@ int type_size(int32_t type) {
     }
 }
 
+// Arenas of an engine's lanes together hold at most this, and an eighth of the
+// device budget.
+constexpr uint64_t ARENA_MAX = 2ull << 30;
+
+static uint64_t arena_limit(const Budget& b) { return std::min(ARENA_MAX, b.cap / 8); }
+
+static uint64_t idle_arenas(const Budget& b) {
+    uint64_t n = 0;
+    for (const Lane* l : b.lanes)
+        if (!l->busy) n += l->arena_bytes;
+    return n;
+}
+
+// The functions below hold the budget's mutex.  An idle lane's work has
+// finished, so its arena can be freed on its stream from any thread.
+static void free_arena(Budget& b, Lane* l) {
+    cudaFreeAsync(l->arena, l->compute);
+    b.arenas -= l->arena_bytes;
+    l->arena = nullptr;
+    l->arena_bytes = 0;
+}
+
+// Gives idle arenas back until they fit beside the reservations and `excess`
+// further bytes (all: every one).
+static void trim_arenas(Budget& b, uint64_t excess, bool all = false) {
+    for (Lane* l : b.lanes) {
+        if (!l->arena || l->busy) continue;
+        if (!all && b.reserved + excess + idle_arenas(b) <= b.cap && b.arenas <= arena_limit(b)) return;
+        free_arena(b, l);
+    }
+}
+
+void lane_open(tp_engine* e, Lane* lane) {
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    e->budget.lanes.push_back(lane);
+}
+
+void lane_close(tp_engine* e, Lane* lane) {
+    lane_drop_arena(e, lane);
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    auto& v = e->budget.lanes;
+    v.erase(std::remove(v.begin(), v.end(), lane), v.end());
+}
+
+void lane_begin(tp_engine* e, Lane* lane) {
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    lane->busy = true;
+}
+
+void lane_end(tp_engine* e, Lane* lane) {
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    lane->busy = false;
+    trim_arenas(e->budget, 0);   // the cap may be another by now
+}
+
+bool lane_drop_arena(tp_engine* e, Lane* lane) {
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    if (!lane->arena) return false;
+    free_arena(e->budget, lane);
+    return true;
+}
+
+void lane_grow_arena(tp_engine* e, Lane* lane, uint64_t want, uint64_t reserved) {
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    Budget& b = e->budget;
+    const uint64_t excess = want > reserved ? want - reserved : 0;
+    if (want <= lane->arena_bytes || b.arenas - lane->arena_bytes + want > arena_limit(b) ||
+        b.reserved + excess + idle_arenas(b) > b.cap)
+        return;
+    if (lane->arena) free_arena(b, lane);
+    if (cudaMallocAsync(&lane->arena, want, lane->compute) != cudaSuccess) {
+        cudaGetLastError();
+        lane->arena = nullptr;
+        return;
+    }
+    lane->arena_bytes = want;
+    b.arenas += want;
+}
+
+bool lane_over(tp_engine* e, uint64_t excess) {
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    trim_arenas(e->budget, excess);
+    return e->budget.reserved + excess > e->budget.cap;
+}
+
 tp_status reserve(tp_engine* e, uint64_t bytes) {
     std::lock_guard<std::mutex> lk(e->budget.mu);
     if (e->budget.fail_next > 0) {
@@ -50,6 +135,7 @@ tp_status reserve(tp_engine* e, uint64_t bytes) {
                     (unsigned long long)e->budget.cap);
     e->budget.reserved += bytes;
     if (e->budget.reserved > e->budget.peak) e->budget.peak = e->budget.reserved;
+    trim_arenas(e->budget, 0);
     return TP_OK;
 }
 
@@ -61,13 +147,44 @@ void release(tp_engine* e, uint64_t bytes) {
     e->budget.cv.notify_all();
 }
 
+static thread_local bool t_alloc_failed = false;
+
+bool take_alloc_failure() {
+    const bool f = t_alloc_failed;
+    t_alloc_failed = false;
+    return f;
+}
+
+static cudaError_t malloc_async(tp_engine* e, void** p, uint64_t bytes, cudaStream_t st) {
+    {
+        std::lock_guard<std::mutex> lk(e->budget.mu);
+        if (e->budget.fail_allocs > 0 && bytes >= e->budget.fail_alloc_bytes) {
+            --e->budget.fail_allocs;
+            return cudaErrorMemoryAllocation;
+        }
+    }
+    const cudaError_t err = cudaMallocAsync(p, bytes, st);
+    if (err != cudaSuccess) cudaGetLastError();
+    return err;
+}
+
 tp_status dev_alloc(tp_engine* e, void** p, uint64_t bytes, cudaStream_t st) {
-    (void)e;
     *p = nullptr;
     if (bytes == 0) bytes = 256;
-    cudaError_t err = cudaMallocAsync(p, bytes, st);
+    cudaError_t err = malloc_async(e, p, bytes, st);
     if (err != cudaSuccess) {
-        cudaGetLastError();
+        std::vector<cudaStream_t> freed;
+        {
+            std::lock_guard<std::mutex> lk(e->budget.mu);
+            for (const Lane* l : e->budget.lanes)
+                if (!l->busy && l->arena) freed.push_back(l->compute);
+            trim_arenas(e->budget, 0, true);
+        }
+        for (cudaStream_t s : freed) cudaStreamSynchronize(s);
+        if (!freed.empty()) err = malloc_async(e, p, bytes, st);
+    }
+    if (err != cudaSuccess) {
+        t_alloc_failed = true;
         *p = nullptr;
         return fail(TP_E_CUDA, "device allocation of %llu bytes failed: %s", (unsigned long long)bytes,
                     cudaGetErrorString(err));
@@ -238,14 +355,6 @@ bool has_narrow(const tp_table* t) {
     return false;
 }
 
-void lane_drop_arena(tp_engine* e, Lane* lane) {
-    if (!lane->arena) return;
-    cudaFreeAsync(lane->arena, lane->compute);
-    e->arena_total -= lane->arena_bytes;
-    lane->arena = nullptr;
-    lane->arena_bytes = 0;
-}
-
 void dev_free(tp_engine* e, void* p, cudaStream_t st) {
     (void)e;
     if (p) cudaFreeAsync(p, st);
@@ -328,6 +437,7 @@ tp_status tp_init(const tp_config* cfg, tp_engine** out) {
     e->lane0.copy = e->copy;
     e->lane0.spill = e->spill;
     e->lane0.host_words = e->host_words;
+    lane_open(e.get(), &e->lane0);
     *out = e.release();
     return TP_OK;
 }
@@ -338,7 +448,7 @@ void tp_shutdown(tp_engine* e) {
     cudaStreamSynchronize(e->compute);
     cudaStreamSynchronize(e->copy);
     cudaStreamSynchronize(e->spill);
-    lane_drop_arena(e, &e->lane0);
+    lane_close(e, &e->lane0);
     if (e->pool.base) cudaFreeHost(e->pool.base);
     if (e->host_words) cudaFreeHost(e->host_words);
     cudaStreamDestroy(e->copy);
@@ -392,6 +502,7 @@ tp_status tp_set_device_budget(tp_engine* e, uint64_t bytes) {
     {
         std::lock_guard<std::mutex> lk(e->budget.mu);
         e->budget.cap = bytes;
+        trim_arenas(e->budget, 0);
     }
     e->budget.cv.notify_all();
     return TP_OK;
@@ -779,6 +890,14 @@ tp_status tp_debug_fail_next_alloc(tp_engine* e, int32_t n) {
     }
     std::lock_guard<std::mutex> lk(e->budget.mu);
     e->budget.fail_next = n;
+    return TP_OK;
+}
+
+tp_status tp_debug_fail_device_allocs(tp_engine* e, uint64_t min_bytes, int32_t n) {
+    if (!e || n < 0) return fail(TP_E_INVALID, "tp_debug_fail_device_allocs: bad argument");
+    std::lock_guard<std::mutex> lk(e->budget.mu);
+    e->budget.fail_alloc_bytes = min_bytes;
+    e->budget.fail_allocs = n;
     return TP_OK;
 }
 

@@ -75,72 +75,104 @@ int64_t paged_value(const tp_table* t, int c, uint64_t row) {
     return 0;
 }
 
-// Arenas of an engine's lanes together hold at most this, and an eighth of the
-// device budget.
-constexpr uint64_t ARENA_MAX = 2ull << 30;
+// Internal status: the lane's arena and what the execution holds beside it
+// would pass the device budget; the query runs again without an arena.
+constexpr tp_status RETRY_NO_ARENA = -4;
 
 // Device memory of one execution, released together at the end.  It comes from
 // the lane's arena while that lasts, then from the stream-ordered allocator;
-// an execution that needed more leaves a larger arena to the next.  Taking
-// every buffer from the allocator cost a small query about 15 us of calls, and
-// next to large results that the caller still held it re-mapped memory for the
-// larger buffers: 1.0 ms in two of three passes of the 15M-group query.
+// an execution that needed more at once leaves a larger arena to the next.
+// Taking every buffer from the allocator cost a small query about 15 us of
+// calls, and next to large results that the caller still held it re-mapped
+// memory for the larger buffers: 1.0 ms in two of three passes of the 15M-group
+// query.
 struct Scratch {
     tp_engine* e;
     Lane* lane;
     cudaStream_t st;
-    std::vector<void*> ptrs;
     uint64_t reserved = 0;
-    uint64_t at = 0, total = 0;   // arena bytes handed out, bytes asked for
-    Scratch(tp_engine* eng, Lane* l) : e(eng), lane(l), st(l->compute) {}
+    Scratch(tp_engine* eng, Lane* l) : e(eng), lane(l), st(l->compute) { lane_begin(e, lane); }
     tp_status alloc(void** p, uint64_t bytes) {
         const uint64_t b = align256(bytes ? bytes : 1);
-        total += b;
-        if (b <= lane->arena_bytes - at) {
-            *p = (uint8_t*)lane->arena + at;
-            at += b;
-            return TP_OK;
+        uint64_t at = 0;
+        size_t k = 0;
+        while (k < pieces.size() && pieces[k].at - at < b) {   // the first gap that holds b bytes
+            at = pieces[k].at + pieces[k].bytes;
+            ++k;
         }
-        tp_status s = dev_alloc(e, p, bytes, st);
-        if (s != TP_OK && at == 0 && lane->arena) {   // the arena itself may be what is missing
-            lane_drop_arena(e, lane);
-            cudaStreamSynchronize(st);
-            clear_error();
-            s = dev_alloc(e, p, bytes, st);
-        }
-        if (s == TP_OK) ptrs.push_back(*p);
-        return s;
+        if (k == pieces.size() && lane->arena_bytes - at < b) return alloc_apart(p, bytes);
+        pieces.insert(pieces.begin() + (long)k, {at, b});
+        *p = (uint8_t*)lane->arena + at;
+        grew(b);
+        return TP_OK;
     }
-    // Gives one buffer back early, ordered on stream s; the arena's wait for the end.
+    // Never from the arena: for buffers that are given back on another stream,
+    // where the arena's next use of their bytes would not be ordered after them.
+    tp_status alloc_apart(void** p, uint64_t bytes) {
+        const uint64_t b = align256(bytes ? bytes : 1);
+        if (over(b)) return RETRY_NO_ARENA;
+        tp_status s = dev_alloc(e, p, bytes, st);
+        if (s) return s;
+        apart.push_back({*p, b});
+        apart_bytes += b;
+        grew(b);
+        return TP_OK;
+    }
+    // Gives one buffer back early, ordered on stream s (the arena's: on the lane's
+    // compute stream, which every use of its bytes is ordered on or after).
     void drop(void* p, cudaStream_t s) {
-        auto it = std::find(ptrs.begin(), ptrs.end(), p);
-        if (it == ptrs.end()) return;
-        dev_free(e, p, s);
-        ptrs.erase(it);
+        for (size_t k = 0; k < apart.size(); ++k) {
+            if (apart[k].first != p) continue;
+            dev_free(e, p, s);
+            apart_bytes -= apart[k].second;
+            live -= apart[k].second;
+            apart.erase(apart.begin() + (long)k);
+            return;
+        }
+        const uint64_t at = (uint64_t)((uint8_t*)p - (uint8_t*)lane->arena);
+        for (size_t k = 0; k < pieces.size(); ++k) {
+            if (pieces[k].at != at) continue;
+            live -= pieces[k].bytes;
+            pieces.erase(pieces.begin() + (long)k);
+            return;
+        }
+    }
+    // Do the arena and the buffers beside it (with `more` bytes to come) hold more
+    // than was reserved for them, and does that pass the budget?
+    bool over(uint64_t more = 0) {
+        const uint64_t held = lane->arena_bytes + apart_bytes + more;
+        return lane->arena && held > reserved && lane_over(e, held - reserved);
     }
     void free_all() {
-        for (void* p : ptrs) dev_free(e, p, st);
-        ptrs.clear();
+        for (auto& a : apart) dev_free(e, a.first, st);
+        apart.clear();
+        pieces.clear();
         if (reserved) release(e, reserved);
-        reserved = 0;
-        const uint64_t want = (total + (1ull << 21) - 1) >> 21 << 21;
-        total = at = 0;
-        uint64_t held = 0, cap = 0;
-        if (want <= lane->arena_bytes || tp_budget_query(e, &held, &cap) != TP_OK) return;
-        if ((e->arena_total += want) - lane->arena_bytes > std::min(ARENA_MAX, cap / 8)) {
-            e->arena_total -= want;   // counted first: other lanes grow theirs at the same time
-            return;
-        }
-        lane_drop_arena(e, lane);
-        if (cudaMallocAsync(&lane->arena, want, st) != cudaSuccess) {
-            cudaGetLastError();
-            lane->arena = nullptr;
-            e->arena_total -= want;
-            return;
-        }
-        lane->arena_bytes = want;
+        reserved = apart_bytes = live = 0;
     }
-    ~Scratch() { free_all(); }
+    // The end of an execution that succeeded.
+    void finish() {
+        for (auto& a : apart) dev_free(e, a.first, st);
+        apart.clear();
+        lane_grow_arena(e, lane, (peak + (1ull << 21) - 1) >> 21 << 21, reserved);
+        free_all();
+    }
+    ~Scratch() {
+        free_all();
+        lane_end(e, lane);
+    }
+
+private:
+    struct Piece {
+        uint64_t at, bytes;
+    };
+    std::vector<Piece> pieces;                        // of the arena, in order
+    std::vector<std::pair<void*, uint64_t>> apart;    // buffers of the allocator
+    uint64_t apart_bytes = 0, live = 0, peak = 0;     // peak: most bytes held at once
+    void grew(uint64_t b) {
+        live += b;
+        peak = std::max(peak, live);
+    }
 };
 
 struct ExecState {
@@ -667,6 +699,18 @@ tp_status alloc_result(tp_engine* e, tp_plan* p, uint64_t cap, tp_result** out, 
 
 namespace {
 
+// Output arrays of an execution, for cap groups.
+tp_status exec_result(ExecState& S, Scratch& sc, uint64_t cap, tp_result** out, tpk::OutDev* od,
+                      unsigned long long* n_groups_dev) {
+    tp_status s = alloc_result(S.e, S.p, cap, out, od, n_groups_dev, S.lane->compute);
+    if (s == TP_OK && sc.over()) {
+        tp_result_free(*out);
+        *out = nullptr;
+        return RETRY_NO_ARENA;
+    }
+    return s;
+}
+
 // Copies rows [0, n) of every array of src to rows [at, at + n) of dst (both
 // results of the same plan), on the device.
 tp_status copy_result_rows(tp_result* dst, uint64_t at, const tp_result* src, uint64_t n, int n_sum,
@@ -954,9 +998,11 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
         void* mem = nullptr;
         ~Held() {
             if (mem) sc.drop(mem, sc.st);
+            sc.reserved -= bytes;
             release(sc.e, bytes);
         }
     } held{sc, bytes};
+    sc.reserved += bytes;
     tp_status s = sc.alloc(&held.mem, bytes);
     if (s) return s;
     void* mem = held.mem;
@@ -1034,7 +1080,7 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     // ---- the ordered result
     tp_result* r = nullptr;
     tpk::OutDev od;
-    s = alloc_result(e, p, n, &r, &od, nullptr, st);
+    s = exec_result(S, sc, n, &r, &od, nullptr);
     if (s == TP_E_BUDGET) return NO_RECORDS;   // the table's own path can split the key range
     if (s) return s;
     std::unique_ptr<tp_result, void (*)(tp_result*)> guard(r, tp_result_free);
@@ -1494,7 +1540,7 @@ tp_status part_spill_fact(ExecState& S, Scratch& sc, PartJoin& pj, const tpk::Qu
         enc_w[c] = narrow ? (uint8_t)frame_width(S.fact->cmin[c], S.fact->cmax[c], full) : 0;
         enc_base[c] = S.fact->cmin[c];
         width[c] = enc_w[c] ? enc_w[c] : full;
-        tp_status s = sc.alloc(&out[c], align256(total * (uint64_t)width[c]));
+        tp_status s = sc.alloc_apart(&out[c], align256(total * (uint64_t)width[c]));   // dropped on the spill stream
         if (s) return s;
         cols.src[cols.n] = colptr[c];
         cols.dst[cols.n] = out[c];
@@ -1968,6 +2014,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
     est -= agg_est;   // the global table is reserved per key range
     if ((s = reserve(e, est))) return s;
     sc.reserved += est;
+    if (sc.over()) return RETRY_NO_ARENA;
     // ---- lookahead filter (Section 5): with a dimension predicate, when the
     // join table would not stay in L2 or the join is partitioned (or asked
     // for); tables shared through the cache go without.  Optional: when its
@@ -2161,7 +2208,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
         }
         if (s) return s;
         tpk::OutDev od;
-        if ((s = alloc_result(e, p, G, &res, &od, S.counters + 1, st))) return s;
+        if ((s = exec_result(S, sc, G, &res, &od, S.counters + 1))) return s;
         std::unique_ptr<tp_result, void (*)(tp_result*)> guard(res, tp_result_free);
         // a small result's rows come back with the status
         tpk::HostMirror m{S.err, lane->host_words, (const unsigned char*)res->dev, nullptr};
@@ -2193,7 +2240,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             if (s != TP_OK && s != NO_RECORDS) return s;
             if (s == TP_OK) {
                 p->history_groups = res->n_groups;
-                sc.free_all();
+                sc.finish();
                 *out = res;
                 return TP_OK;
             }
@@ -2235,10 +2282,10 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             tp_result* r = nullptr;
             tpk::OutDev od;
             auto alloc_rows = [&]() {   // the extrapolated capacity, else just the rows needed
-                tp_status t = alloc_result(e, p, want, &r, &od, nullptr, st);
+                tp_status t = exec_result(S, sc, want, &r, &od, nullptr);
                 if (t == TP_E_BUDGET && want > need_rows) {
                     want = need_rows;
-                    t = alloc_result(e, p, want, &r, &od, nullptr, st);
+                    t = exec_result(S, sc, want, &r, &od, nullptr);
                 }
                 return t;
             };
@@ -2463,17 +2510,19 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
         res->n_groups = res_at;
         p->history_groups = res_at;
     }
-    sc.free_all();
+    sc.finish();
     *out = res;
     return TP_OK;
 }
 
 tp_status execute_locked(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out) {
+    take_alloc_failure();
     for (;;) {   // Section 3.3.2: a task retried with a better estimate
         const tp_status s = execute_once(p, lane, cache, out);
         if (s == RETRY_UNPACKED) p->no_packed = true;   // neither comes back once its estimate is dropped
         else if (s == RETRY_FANOUT) p->fan = 0;
-        else return s;
+        else if (s == RETRY_NO_ARENA) lane_drop_arena(p->eng, lane);
+        else if (!(take_alloc_failure() && s == TP_E_CUDA && lane_drop_arena(p->eng, lane))) return s;
         p->eng->retries++;
     }
 }

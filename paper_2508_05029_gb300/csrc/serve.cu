@@ -749,6 +749,8 @@ void completer(tp_server* sv) {
 void server_free(tp_server* sv) {
     if (!sv) return;
     cudaSetDevice(sv->e->device);
+    for (Lane& l : sv->lanes) lane_close(sv->e, &l);
+    lane_close(sv->e, &sv->dlane);
     sv->lanes.push_back(sv->dlane);   // freed with the others below
     for (Lane& l : sv->lanes) {
         if (l.compute) cudaStreamSynchronize(l.compute);
@@ -762,7 +764,6 @@ void server_free(tp_server* sv) {
     cache_evict_idle(sv->e, &sv->cache, 0);
     evict_joins(sv, 0, sv->e->compute);
     for (Lane& l : sv->lanes) {
-        lane_drop_arena(sv->e, &l);
         if (l.compute) cudaStreamDestroy(l.compute);
         if (l.copy) cudaStreamDestroy(l.copy);
         if (l.spill) cudaStreamDestroy(l.spill);
@@ -799,12 +800,14 @@ tp_status tp_server_start(tp_engine* e, int32_t workers, int32_t max_inflight, u
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&l.copy, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&l.spill, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaHostAlloc((void**)&l.host_words, LANE_HOST_BYTES, cudaHostAllocDefault));
+        lane_open(e, &l);
     }
     if (sv->batch_on) {
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&sv->dlane.compute, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&sv->dlane.copy, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaStreamCreateWithFlags(&sv->dlane.spill, cudaStreamNonBlocking));
         TP_TRY_CUDA(cudaHostAlloc((void**)&sv->dlane.host_words, LANE_HOST_BYTES, cudaHostAllocDefault));
+        lane_open(e, &sv->dlane);
         for (Slot& sl : sv->slots) {
             TP_TRY_CUDA(cudaStreamCreateWithFlags(&sl.st, cudaStreamNonBlocking));
             TP_TRY_CUDA(cudaEventCreateWithFlags(&sl.ev, cudaEventDisableTiming));

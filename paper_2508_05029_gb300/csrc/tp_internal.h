@@ -50,6 +50,12 @@ struct PagePool {
 // Reservations before execution (Section 3.3.2): a task states its device
 // bytes up front; a reservation that does not fit under the cap fails instead
 // of running into out-of-memory mid-way.
+//
+// Arenas (below) are memory besides the reservations.  reserve() gives idle
+// lanes' arenas back when they and the reservations would pass the cap
+// together, and the executions of a lane whose own arena would pass it run
+// without one (lane_over).
+struct Lane;
 struct Budget {
     std::mutex mu;
     std::condition_variable cv;
@@ -57,6 +63,12 @@ struct Budget {
     uint64_t reserved = 0;
     uint64_t peak = 0;
     int fail_next = 0;
+    std::vector<Lane*> lanes;     // every open lane
+    uint64_t arenas = 0;          // bytes of their arenas
+    // injected failures of device allocations: the next fail_allocs of at
+    // least fail_alloc_bytes
+    int fail_allocs = 0;
+    uint64_t fail_alloc_bytes = 0;
 };
 
 // A contiguous piece of one column inside one page.
@@ -104,6 +116,7 @@ struct Lane {
     // (stream-ordered on compute: an execution starts after the one before)
     void* arena = nullptr;
     uint64_t arena_bytes = 0;
+    bool busy = false;            // an execution uses it (under the budget's mutex)
 };
 constexpr uint64_t LANE_WORD_BYTES = 4096;
 constexpr uint64_t LANE_HOST_BYTES = LANE_WORD_BYTES + (128u << 10);
@@ -127,7 +140,6 @@ struct tp_engine {
     std::atomic<uint64_t> h2d_bytes{0}, d2h_bytes{0}, batches{0}, launches{0}, retries{0};
     std::atomic<uint64_t> jit_compiles{0}, jit_failures{0}, jit_launches{0}, jit_us{0};
     std::atomic<uint64_t> split_passes{0}, lip_filters{0};
-    std::atomic<uint64_t> arena_total{0};   // bytes of all lanes' arenas
     // small pinned scratch for status words read back after an execution
     uint64_t* host_words = nullptr;
     tp::Lane lane0;                  // compute, copy, host_words of the engine itself
@@ -365,10 +377,26 @@ int batch_kernel_grid(const void* jit_kernel_or_null, uint32_t smem_bytes, int n
 tp_status alloc_result(tp_engine* e, tp_plan* p, uint64_t cap, tp_result** out, tpk::OutDev* od,
                        unsigned long long* n_groups_dev, cudaStream_t st);
 
-// Gives a lane's arena back (its work has finished or is ordered before).
-void lane_drop_arena(tp_engine* e, Lane* lane);
-// device memory (stream-ordered allocator on the compute stream)
+// A lane from its set-up to its end (which gives its arena back).
+void lane_open(tp_engine* e, Lane* lane);
+void lane_close(tp_engine* e, Lane* lane);
+// An execution on the lane: its arena is not taken away meanwhile.
+void lane_begin(tp_engine* e, Lane* lane);
+void lane_end(tp_engine* e, Lane* lane);
+// Gives a lane's arena back (its work has finished or is ordered before);
+// false: it has none.
+bool lane_drop_arena(tp_engine* e, Lane* lane);
+// A larger arena for the next execution of a busy lane whose present one held
+// `reserved` bytes of the budget, if the limits allow it.
+void lane_grow_arena(tp_engine* e, Lane* lane, uint64_t want, uint64_t reserved);
+// Would `excess` bytes besides the reservations pass the cap?  Idle arenas make
+// room first.
+bool lane_over(tp_engine* e, uint64_t excess);
+// device memory (stream-ordered allocator on the compute stream); a failure
+// gives the idle arenas back and tries once more
 tp_status dev_alloc(tp_engine* e, void** p, uint64_t bytes, cudaStream_t st);
+// Has dev_alloc failed on this thread since the last call?
+bool take_alloc_failure();
 void dev_free(tp_engine* e, void* p, cudaStream_t st);
 
 }  // namespace tp

@@ -154,6 +154,7 @@ SIGNATURES = {
     "tp_last_error": (ctypes.c_char_p, []),
     "tp_stats_get": (_i32, [_vp, ctypes.POINTER(tp_stats)]),
     "tp_debug_fail_next_alloc": (_i32, [_vp, _i32]),
+    "tp_debug_fail_device_allocs": (_i32, [_vp, _u64, _i32]),
     "tp_debug_pack_bits": (_i32, [_vp, _u64, _i32, _vp]),
     "tp_batch_create": (_i32, [_vp, _PP, _i32, ctypes.c_char_p, _PP]),
     "tp_batch_execute": (_i32, [_vp, _PP]),
@@ -258,6 +259,9 @@ class Engine:
 
     def fail_next_alloc(self, n: int):
         _check(self.lib.tp_debug_fail_next_alloc(self.h, n))
+
+    def fail_device_allocs(self, min_bytes: int, n: int):
+        _check(self.lib.tp_debug_fail_device_allocs(self.h, min_bytes, n))
 
     # tables ---------------------------------------------------------------
     def _desc(self, names, dtypes, batch_rows=0):
