@@ -246,12 +246,15 @@ struct KernelTimer {
         ev.clear();
         rows = 0;
     }
-    ~KernelTimer() {
+    void discard() {  // an attempt that is not counted
         for (auto& p : ev) {
             cudaEventDestroy(p.first);
             cudaEventDestroy(p.second);
         }
+        ev.clear();
+        rows = 0;
     }
+    ~KernelTimer() { discard(); }
 };
 
 tpk::DevCol devcol(const tp_table* t, int c, const void* ptr) {
@@ -1004,7 +1007,8 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     } held{sc, bytes};
     sc.reserved += bytes;
     tp_status s = sc.alloc(&held.mem, bytes);
-    if (s) return s;
+    if (s == RETRY_NO_ARENA) return s;
+    if (s) return NO_RECORDS;   // the table needs less memory
     void* mem = held.mem;
     uint8_t* at = (uint8_t*)mem;
     rec.r0 = (uint4*)at;
@@ -1070,7 +1074,7 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     const uint32_t err = (uint32_t)S.lane->host_words[0];
     if ((s = map_err(err))) return s;
     if (err & tpk::ERR_RECORDS) {
-        timer.ev.clear();   // a discarded attempt is not counted
+        timer.discard();
         p->no_records = true;
         e->retries++;
         TP_TRY_CUDA(cudaMemsetAsync(S.err, 0, 4, st));
@@ -1081,7 +1085,10 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     tp_result* r = nullptr;
     tpk::OutDev od;
     s = exec_result(S, sc, n, &r, &od, nullptr);
-    if (s == TP_E_BUDGET) return NO_RECORDS;   // the table's own path can split the key range
+    if (s == TP_E_BUDGET || s == TP_E_CUDA) {   // the table's own path can split the key range
+        timer.discard();
+        return NO_RECORDS;
+    }
     if (s) return s;
     std::unique_ptr<tp_result, void (*)(tp_result*)> guard(r, tp_result_free);
     TP_TRY_CUDA(tpk::launch_rec_emit(rec, ns, n_groups, offsets, od, e->num_sms, st));
@@ -2433,7 +2440,7 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
             const uint32_t err = (uint32_t)lane->host_words[0];
             if ((s = map_err(err))) return s;
             if (err & tpk::ERR_OVERFLOW) {
-                timer.ev.clear();  // a discarded attempt is not counted
+                timer.discard();
                 if (++attempt > 6) return fail(TP_E_INTERNAL, "aggregation table overflow after retries");
                 // retry with a table sized from what was seen so far (Section 3.3.2:
                 // a task that ran out of memory is retried with a better estimate);

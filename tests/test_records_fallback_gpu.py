@@ -1,0 +1,75 @@
+"""Many-group aggregation when its records cannot be had or did not suit the
+plan: the query runs through the global table, and a later execution takes the
+records again.  A record scan is a run-time compiled launch, the global table's
+kernels are not."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2508_05029_gb300 import theseus as T
+from tests.helpers import assert_matches_oracle
+
+pytestmark = pytest.mark.gpu
+ROWS = (4 << 20) + 1025
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2508_05029_gb300 import build
+    build.build()
+
+
+class Case:
+    """A plan over rows of (key, a); each run is checked and says what it launched."""
+
+    def __init__(self, fact, q, **kw):
+        self.fact, self.q, self.e = fact, q, T.Engine(**kw)
+        self.dev = {k: torch.from_numpy(v).cuda() for k, v in fact.items()}
+        self.table = self.e.table_from_torch(self.dev)
+        torch.cuda.synchronize()
+        self.plan = self.e.plan(self.table, None, q)
+        self.ref = oracle.run_query(fact, None, q)
+
+    def change(self, key):
+        self.fact["key"][:] = key
+        self.dev["key"].copy_(torch.from_numpy(key).cuda())
+        torch.cuda.synchronize()
+        self.ref = oracle.run_query(self.fact, None, self.q)
+
+    def run(self):
+        """(record scans, retries) of one execution"""
+        s0 = self.e.stats()
+        with self.plan.execute() as r:
+            assert_matches_oracle(r, self.ref, self.q["aggs"])
+        s1 = self.e.stats()
+        return s1["jit_launches"] - s0["jit_launches"], s1["retries"] - s0["retries"]
+
+
+def _query(flt=None):
+    return dict(filter=flt, join=None, group=[("fact", "key", 64)], aggs=[("sum", "a"), ("count",)])
+
+
+def _fact(key, seed=1):
+    return dict(key=np.ascontiguousarray(key, np.int64), a=np.random.default_rng(seed).integers(-10**9, 10**9, len(key)))
+
+
+@pytest.fixture
+def case():
+    made = []
+
+    def make(*a, **kw):
+        made.append(Case(*a, **kw))
+        return made[-1]
+    yield make
+    for c in made:
+        c.e.close()
+
+
+def test_records_that_cannot_be_allocated(case):
+    rng = np.random.default_rng(3)
+    c = case(_fact(rng.integers(0, 1 << 20, ROWS)), _query())
+    c.e.fail_device_allocs(64 * MB, 1)     # the records take about 90 MB, the table 32
+    assert c.run() == (0, 0)
+    assert c.run() == (1, 0)
