@@ -887,7 +887,7 @@ constexpr tp_status NO_RECORDS = -2;
 bool records_usable(const ExecState& S) {
     const tp_plan* p = S.p;
     const tp_plan_desc& d = p->d;
-    if (p->no_records || (S.e->cfg.flags & (TP_FLAG_NO_STAGED | TP_FLAG_EXACT_ONLY | TP_FLAG_NO_DIRECT_AGG)) ||
+    if ((S.e->cfg.flags & (TP_FLAG_NO_STAGED | TP_FLAG_EXACT_ONLY | TP_FLAG_NO_DIRECT_AGG)) ||
         S.fact->placement == PL_PAGES || S.fact->rows < REC_MIN_ROWS || S.fact->rows >= (1ull << 32) ||
         p->n_dims > 1 || d.join_many || d.n_group == 0 || p->n_sum > tpk::REC_MAX_SUM)
         return false;
@@ -940,7 +940,7 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     cudaStream_t st = S.lane->compute;
     const int ns = p->n_sum;
     const uint64_t rows = S.fact->rows;
-    if (std::min(rspan, groups) < REC_MIN_GROUPS) return NO_RECORDS;
+    if (std::min(rspan, groups) < REC_MIN_GROUPS || groups <= p->no_records_groups) return NO_RECORDS;
     // a dense range: partitions that shared memory addresses directly (two
     // CTAs per SM), otherwise hashed ones at 0.45 of their table's slots; also
     // when the groups fill less than an eighth of the range, where looking
@@ -1075,7 +1075,8 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     if ((s = map_err(err))) return s;
     if (err & tpk::ERR_RECORDS) {
         timer.discard();
-        p->no_records = true;
+        p->no_records_groups = groups;
+        p->rec_skew = -1.0;   // the rows may lie otherwise by now
         e->retries++;
         TP_TRY_CUDA(cudaMemsetAsync(S.err, 0, 4, st));
         return NO_RECORDS;

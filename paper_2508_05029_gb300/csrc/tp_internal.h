@@ -195,7 +195,9 @@ struct tp_plan {
     int gdim[4] = {-1, -1, -1, -1};                 // dimension of group field g, -1: fact
     uint64_t distinct_groups = 0;   // estimated distinct group keys of the fact table, 0 until measured
     double rec_skew = -1.0;         // sampled: fullest key partition over the mean, < 0 until measured
-    bool no_records = false;        // a record partition overflowed: the global table from then on
+    // group estimate at which a record partition overflowed (0: none has): the
+    // global table until an estimate is larger
+    uint64_t no_records_groups = 0;
     // run-time compiled kernels by the bytes of their shape and geometry
     std::vector<std::pair<std::string, const void*>> kernels;
     bool no_packed = false;      // a packed join table could not place a key: unpacked ones from then on

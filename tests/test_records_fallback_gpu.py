@@ -73,3 +73,20 @@ def test_records_that_cannot_be_allocated(case):
     c.e.fail_device_allocs(64 * MB, 1)     # the records take about 90 MB, the table 32
     assert c.run() == (0, 0)
     assert c.run() == (1, 0)
+
+
+def test_records_come_back_after_an_overflow(case):
+    """A quarter of the 1,024 partitions made for 1.8 million groups gets 4,700
+    keys, more than their tables hold; the next execution knows of 3.7 million
+    groups and makes twice as many partitions."""
+    rng = np.random.default_rng(4)
+    key = rng.integers(0, 2_100_000, ROWS) * 4_090
+    key[0], key[1] = 1 << 33, 0
+    c = case(_fact(key), _query())
+    assert c.run() == (1, 0)
+    keys = np.concatenate([(p << 23) + np.arange(4_700 if p % 4 == 0 else 3_255) * 1_700 for p in range(1024)])
+    key = rng.permutation(np.concatenate([[1 << 33], keys, rng.choice(keys, ROWS - 1 - len(keys))]))
+    c.change(key)
+    assert c.run() == (1, 1)       # through the table in the end
+    assert c.run() == (1, 0)
+    assert c.run() == (1, 0)
