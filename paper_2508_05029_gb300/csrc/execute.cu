@@ -966,8 +966,10 @@ tp_status aggregate_records(ExecState& S, Scratch& sc, KernelTimer& timer, uint6
     rec.shift = shift;
     rec.n_part = (uint32_t)(((rspan - 1) >> shift) + 1);
     const tpk::QueryDev q = fact_query(S);
-    // ---- how evenly the passing rows spread, sampled once per plan
-    if (p->rec_skew < 0) {
+    // ---- how evenly the passing rows spread over these partitions, sampled once
+    if (p->rec_skew < 0 || p->rec_parts != rec.n_part || p->rec_shift != shift) {
+        p->rec_parts = rec.n_part;
+        p->rec_shift = shift;
         void* hist = nullptr;
         tp_status hs = sc.alloc(&hist, ((uint64_t)rec.n_part + 1) * 4);
         if (hs) return hs;

@@ -194,7 +194,11 @@ struct tp_plan {
     double dim_sel[4] = {-1.0, -1.0, -1.0, -1.0};   // sampled predicate pass rates
     int gdim[4] = {-1, -1, -1, -1};                 // dimension of group field g, -1: fact
     uint64_t distinct_groups = 0;   // estimated distinct group keys of the fact table, 0 until measured
-    double rec_skew = -1.0;         // sampled: fullest key partition over the mean, < 0 until measured
+    // sampled: fullest key partition over the mean, < 0 until measured, and the
+    // partitions it was measured for
+    double rec_skew = -1.0;
+    uint32_t rec_parts = 0;
+    int rec_shift = 0;
     // group estimate at which a record partition overflowed (0: none has): the
     // global table until an estimate is larger
     uint64_t no_records_groups = 0;

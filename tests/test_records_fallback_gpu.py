@@ -90,3 +90,17 @@ def test_records_come_back_after_an_overflow(case):
     assert c.run() == (1, 1)       # through the table in the end
     assert c.run() == (1, 0)
     assert c.run() == (1, 0)
+
+
+def test_evenness_is_sampled_for_the_partitions_in_use(case):
+    """Keys in every second range of 2^13: uneven over the partitions of that
+    width that the first estimate asks for, even over the wider ones that the
+    measured group count does."""
+    rng = np.random.default_rng(5)
+    pool = np.arange(1 << 24).reshape(-1, 1 << 13)[::2].ravel()
+    key = rng.choice(rng.choice(pool, 300_000, replace=False), ROWS)
+    key[0], key[1] = 0, (1 << 24) - 1
+    c = case(_fact(key), _query())
+    assert c.run() == (0, 0)
+    assert c.run() == (1, 0)
+    assert c.run() == (1, 0)
