@@ -904,14 +904,16 @@ tpk::QueryDev fact_query(const ExecState& S) {
     return make_query(S, colptr);
 }
 
-// p->distinct_groups from HyperLogLog registers over every fact row's key.
+// p->distinct_groups from HyperLogLog registers over the passing rows' keys.
 tp_status estimate_distinct(ExecState& S, Scratch& sc) {
     cudaStream_t st = S.lane->compute;
     void* regs = nullptr;
     tp_status s = sc.alloc(&regs, tpk::HLL_REGS * 4);
     if (s) return s;
     TP_TRY_CUDA(cudaMemsetAsync(regs, 0, tpk::HLL_REGS * 4, st));
-    TP_TRY_CUDA(tpk::launch_rec_distinct(fact_query(S), S.fact->rows, (uint32_t*)regs, S.e->num_sms, st));
+    tpk::QueryDev q = fact_query(S);
+    if (S.p->selectivity >= 0.9) q.has_filter = 0;   // not worth reading its column
+    TP_TRY_CUDA(tpk::launch_rec_distinct(q, S.fact->rows, (uint32_t*)regs, S.e->num_sms, st));
     mark_launch(S.e);
     std::vector<uint32_t> h(tpk::HLL_REGS);
     TP_TRY_CUDA(cudaMemcpyAsync(h.data(), regs, tpk::HLL_REGS * 4, cudaMemcpyDeviceToHost, st));
@@ -1896,9 +1898,12 @@ tp_status execute_once(tp_plan* p, Lane* lane, DimCache* cache, tp_result** out)
         if (groups == 0) {
             groups = (uint64_t)std::ceil(S.fact->rows * std::min(1.0, p->selectivity * 1.25)) + 16;
             if (p->key_bits < 40) groups = std::min<uint64_t>(groups, 1ull << p->key_bits);
-            // sparse keys: the rows bound the groups loosely, a table for that
-            // many costs more than counting the distinct keys once per plan
-            if (records_usable(S) && (!have_range || rspan > 4 * std::max<uint64_t>(groups, DIRECT_AGG_ALWAYS))) {
+            // sparse keys: the rows bound the groups loosely, and a table for that
+            // many costs more than counting the distinct keys once per plan when it
+            // is larger than the keys themselves (not under a selective filter: 1%
+            // of 60M rows need 64 MB, the count reads 480)
+            if (records_usable(S) && (!have_range || rspan > 4 * std::max<uint64_t>(groups, DIRECT_AGG_ALWAYS)) &&
+                pow2_at_least((uint64_t)std::ceil(groups / lf)) * words > S.fact->rows) {
                 if (p->distinct_groups == 0 && (s = estimate_distinct(S, sc))) return s;
                 groups = std::min<uint64_t>(groups, p->distinct_groups + p->distinct_groups / 8 + 1024);
             }

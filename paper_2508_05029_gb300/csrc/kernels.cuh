@@ -482,7 +482,7 @@ cudaError_t launch_rec_emit(const RecDev& rec, int n_sum, const uint32_t* groups
 // the most of them in one partition; hist: n_part + 1 zeroed words.
 cudaError_t launch_rec_sample(const QueryDev& q, uint64_t n, uint32_t samples, const RecDev& rec,
                               uint32_t* hist, unsigned long long* out, cudaStream_t st);
-// HyperLogLog registers (HLL_REGS words, zeroed) of the rows' group keys.
+// HyperLogLog registers (HLL_REGS words, zeroed) of the passing rows' group keys.
 cudaError_t launch_rec_distinct(const QueryDev& q, uint64_t n, uint32_t* regs, int num_sms, cudaStream_t st);
 
 // ------------------------------------------------------- partitioned join

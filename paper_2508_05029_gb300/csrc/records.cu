@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(RSAMPLE_THREADS)
     }
 }
 
-// Distinct group keys, by HyperLogLog (Flajolet et al. 2007) over 2^12
+// Distinct group keys of the rows that pass the filter, by HyperLogLog (Flajolet et al. 2007) over 2^12
 // registers: the top bits of a key's hash pick a register, which keeps the
 // longest run of leading zeros of the rest, plus one.
 __global__ void __launch_bounds__(REC_THREADS)
@@ -550,6 +550,15 @@ __global__ void __launch_bounds__(REC_THREADS)
     for (uint64_t r = ((uint64_t)blockIdx.x * REC_THREADS + threadIdx.x) * 4; r < n;
          r += (uint64_t)gridDim.x * REC_THREADS * 4) {
         uint64_t key[4] = {0, 0, 0, 0};
+        uint32_t pm = 15u;
+        if (q.has_filter) {
+            int64_t f[4];
+            ld_quad_n(q.fcol, r, n, f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (f[i] < q.flo || f[i] > q.fhi) pm &= ~(1u << i);
+            if (pm == 0) continue;
+        }
         for (int g = 0; g < q.n_group; ++g) {
             int64_t v[4];
             ld_quad_n(q.gcol[g], r, n, v);
@@ -558,7 +567,7 @@ __global__ void __launch_bounds__(REC_THREADS)
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            if (r + i >= n || (i > 0 && key[i] == key[i - 1])) continue;
+            if (r + i >= n || !(pm >> i & 1u) || (i > 0 && (pm >> (i - 1) & 1u) && key[i] == key[i - 1])) continue;
             const uint64_t h = fmix64(key[i]);
             const uint32_t z = (uint32_t)__clzll((long long)(h << HLL_BITS | 1ull << (HLL_BITS - 1))) + 1u;
             uint32_t* w = sm + (h >> (64 - HLL_BITS));

@@ -193,7 +193,7 @@ struct tp_plan {
     tp_filter dflt[4] = {};
     double dim_sel[4] = {-1.0, -1.0, -1.0, -1.0};   // sampled predicate pass rates
     int gdim[4] = {-1, -1, -1, -1};                 // dimension of group field g, -1: fact
-    uint64_t distinct_groups = 0;   // estimated distinct group keys of the fact table, 0 until measured
+    uint64_t distinct_groups = 0;   // estimated distinct group keys of the passing rows, 0 until measured
     // sampled: fullest key partition over the mean, < 0 until measured, and the
     // partitions it was measured for
     double rec_skew = -1.0;

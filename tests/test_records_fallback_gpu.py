@@ -104,3 +104,38 @@ def test_evenness_is_sampled_for_the_partitions_in_use(case):
     assert c.run() == (0, 0)
     assert c.run() == (1, 0)
     assert c.run() == (1, 0)
+
+
+HLL_BYTES = 4 * 4096
+
+
+def _first(c):
+    s0 = c.e.stats()["d2h_bytes"]
+    r = c.plan.execute()
+    read = c.e.stats()["d2h_bytes"] - s0
+    assert_matches_oracle(r, c.ref, c.q["aggs"])
+    r.free()
+    return read
+
+
+@pytest.mark.parametrize("sel,counts", [(0.01, False), (0.2, True), (1.0, True)])
+def test_distinct_keys_are_counted_where_the_rows_say_too_little(case, sel, counts):
+    """Not under a selective filter, whose rows bound the groups better than a pass
+    over every key is worth."""
+    rng = np.random.default_rng(6)
+    fact = _fact(rng.integers(0, 2_000_000, ROWS) * 1_000_003)
+    fact["d"] = rng.integers(0, 1000, ROWS).astype(np.int32)
+    c = case(fact, _query(dict(col="d", lo=0, hi=int(1000 * sel) - 1)))
+    assert (_first(c) >= HLL_BYTES) == counts
+
+
+def test_only_keys_that_pass_are_counted(case):
+    """2 million keys, 20,000 of them in the rows that pass: the first execution's
+    table is one for 20,000 groups."""
+    rng = np.random.default_rng(7)
+    d = rng.integers(0, 1000, ROWS).astype(np.int32)
+    key = np.where(d < 200, rng.integers(0, 20_000, ROWS), rng.integers(0, 2_000_000, ROWS)) * 1_000_003
+    fact = dict(_fact(key), d=d)
+    c = case(fact, _query(dict(col="d", lo=0, hi=199)))
+    assert _first(c) >= HLL_BYTES
+    assert c.e.stats()["peak_reserved"] < 64 * MB
