@@ -861,9 +861,13 @@ const void* plan_kernel(tp_plan* p, const tpk::QueryDev& q, const int8_t* mode, 
         put(mode[s]);
         put(narrow[s]);
     }
-    for (auto& k : p->kernels)
-        if (k.first == key) return k.second;
+    {
+        std::lock_guard<std::mutex> lk(p->kernels_mu);
+        for (auto& k : p->kernels)
+            if (k.first == key) return k.second;
+    }
     const void* k = compile();
+    std::lock_guard<std::mutex> lk(p->kernels_mu);
     if (k) p->kernels.emplace_back(key, k);
     return k;
 }

@@ -202,7 +202,9 @@ struct tp_plan {
     // group estimate at which a record partition overflowed (0: none has): the
     // global table until an estimate is larger
     uint64_t no_records_groups = 0;
-    // run-time compiled kernels by the bytes of their shape and geometry
+    // run-time compiled kernels by the bytes of their shape and geometry; a
+    // server's lane and tp_execute may run the plan at the same time
+    std::mutex kernels_mu;
     std::vector<std::pair<std::string, const void*>> kernels;
     bool no_packed = false;      // a packed join table could not place a key: unpacked ones from then on
     // fan-out: most build rows of one key an execution met (0: none has counted
