@@ -177,6 +177,23 @@ Request* pick(tp_server* sv) {
     return nullptr;
 }
 
+uint64_t evict_joins(tp_server* sv, uint64_t need, cudaStream_t st);
+
+// One execution on a lane; where the budget refuses it, once more after what
+// the server keeps but nobody uses is freed (cached dimension tables, join
+// tables of batched requests).
+tp_status run_on_lane(tp_server* sv, tp_plan* p, Lane* lane, tp_result** res) {
+    DimCache* cache = sv->cache_on ? &sv->cache : nullptr;
+    tp_status st = execute_on_lane(p, lane, cache, res);
+    if (st != TP_E_BUDGET) return st;
+    bool freed = cache && cache_evict_idle(sv->e, cache, 0) > 0;
+    {
+        std::lock_guard<std::mutex> lk(sv->mu);
+        freed = evict_joins(sv, 0, lane->compute) > 0 || freed;
+    }
+    return freed ? execute_on_lane(p, lane, cache, res) : st;
+}
+
 void worker(tp_server* sv, int idx) {
     Lane& lane = sv->lanes[idx];
     cudaSetDevice(sv->e->device);
@@ -199,10 +216,7 @@ void worker(tp_server* sv, int idx) {
             c0 = sv->completions;   // completions before this attempt
         }
         tp_result* res = nullptr;
-        DimCache* cache = sv->cache_on ? &sv->cache : nullptr;
-        tp_status st = execute_on_lane(r->plan, &lane, cache, &res);
-        if (st == TP_E_BUDGET && cache && cache_evict_idle(sv->e, cache, 0) > 0)
-            st = execute_on_lane(r->plan, &lane, cache, &res);
+        tp_status st = run_on_lane(sv, r->plan, &lane, &res);
         // the execution synchronised its lane; the result's memory may be freed
         // on the engine's stream, which outlives the server's lanes
         if (res) res->stream = nullptr;
@@ -578,10 +592,7 @@ void dispatcher(tp_server* sv) {
                 lk.unlock();
                 plan_info(sv, r->plan);   // its shape joins the batched kernel's next compilation
                 tp_result* res = nullptr;
-                DimCache* cache = sv->cache_on ? &sv->cache : nullptr;
-                tp_status st1 = execute_on_lane(r->plan, &sv->dlane, cache, &res);
-                if (st1 == TP_E_BUDGET && cache && cache_evict_idle(e, cache, 0) > 0)
-                    st1 = execute_on_lane(r->plan, &sv->dlane, cache, &res);
+                tp_status st1 = run_on_lane(sv, r->plan, &sv->dlane, &res);
                 if (res) res->stream = nullptr;
                 const std::string msg = st1 ? tp_last_error() : "";
                 lk.lock();
