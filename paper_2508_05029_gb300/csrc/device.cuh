@@ -119,10 +119,11 @@ __device__ __forceinline__ void atomic_add_i128(uint64_t* lo, uint64_t* hi, I128
 // rows test their key before the probe (and before a partitioned join spills
 // them).  With h = fmix64(key), the top bits of h pick one 64-bit word and its
 // low 20 bits two bits in each half of the word.  An insert is one reduction
-// and a test one 8-byte load; at 16 bits per key about one key in 500 passes
-// that was not inserted, and an inserted key always does.  (Eight 32-bit words
-// of 256-bit blocks: eight reductions per insert, two 16-byte loads and twice
-// the instructions per test.)
+// and a test one 8-byte load.  An inserted key always passes; of the others
+// about one in 555 at 24 bits per key, the least a filter below its size limit
+// has for the admitted keys (16 bits: one in 185; 48: one in 3100; counted on
+// 2^18 words).  (Eight 32-bit words of 256-bit blocks: eight reductions per
+// insert, two 16-byte loads and twice the instructions per test.)
 
 __device__ __forceinline__ uint64_t lip_bits(uint32_t h) {
     const uint32_t lo = 1u << (h & 31u) | 1u << (h >> 5 & 31u), hi = 1u << (h >> 10 & 31u) | 1u << (h >> 15 & 31u);

@@ -1782,8 +1782,8 @@ struct JoinSize {
 
 // 64-bit keys take packed buckets when the payload leaves the distance bits
 // and the expected load is at most PACK_MAX_LOAD, where the longest distance
-// measured over 2^12 .. 2^26 slots was 22 buckets (30 can be recorded; at 0.7
-// it was 38).  A dimension predicate's sampled pass rate (4096 rows, three
+// counted in fills of 2^12 .. 2^26 slots with random buckets was 24 (30 can be
+// recorded; at 0.7 it was 52).  A dimension predicate's sampled pass rate (4096 rows, three
 // standard errors up) sizes the table for the admitted rows alone: only packed
 // tables, whose build notices a table that is too small at once.
 constexpr double PACK_MAX_LOAD = 0.6;
