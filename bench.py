@@ -1002,6 +1002,53 @@ def hashed_join_measure(T, W, torch, dev, stream, n_fact, n_dim, peak, reps=10):
     return out
 
 
+# ------------------------------------------------------------------ the line
+LINE_BYTES = 3000   # a line longer than what a reader of the output keeps is lost as a whole
+
+
+def _short(x):
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    return [_short(v) for v in x] if isinstance(x, list) else x
+
+
+def _ms(leg):
+    """A leg's time: its own figure, or the first one inside it."""
+    if not isinstance(leg, dict):
+        return None
+    for k in ("ms_per_step", "ms", "ms_per_query"):
+        if isinstance(leg.get(k), (int, float)):
+            return leg[k]
+    return next((m for m in map(_ms, leg.values()) if m is not None), None)
+
+
+def brief(line):
+    """The line as it is printed: every figure of the headline whole; of the other
+    legs one time each, of the request loops [p50, p99] in ms per rate and the
+    closed loop's queries/s."""
+    out = dict(line)
+    if line.get("e2e"):
+        out["e2e"] = {k: v for k, v in line["e2e"].items() if not isinstance(v, dict)}
+    if line.get("cpu_baseline"):
+        out["cpu_baseline"] = {k: v for k, v in line["cpu_baseline"].items() if not isinstance(v, dict)}
+    out["extra"] = {k: {"ms": _ms(v)} for k, v in (line.get("extra") or {}).items()}
+    pats = {}
+    for name, p in (line.get("patterns") or {}).items():
+        if "batched_ms" in p:
+            pats[name] = {k: p[k] for k in ("batched_ms", "plain_ms") if k in p}
+        else:
+            pats[name] = {k: [v["p50_ms"], v["p99_ms"]] if "p50_ms" in v else v.get("qps")
+                          for k, v in p.items() if isinstance(v, dict)}
+    out["patterns"] = pats or None
+    out = dict(_short(out), value=line["value"], ms_per_step=line["ms_per_step"])
+    for k in ("patterns", "extra"):      # never at the headline's cost
+        if len(json.dumps(out)) > LINE_BYTES:
+            out[k] = "see stderr"
+    return out
+
+
 # ------------------------------------------------------------------ GPU arm
 def main():
     args = parse_args()
@@ -1126,7 +1173,8 @@ def main():
             "e2e": e2e, "gpu_launches": launches, "clocks": clk, "cpu_baseline": cpu, "extra": extra,
             "patterns": patterns,
         }
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)   # every leg's figures
+        print(json.dumps(brief(line)), flush=True)
     barrier(world)
     if world > 1:
         import torch.distributed as dist
