@@ -92,35 +92,42 @@ __device__ __forceinline__ void agg_slots(const AggTable& t, const uint64_t (&ke
             s[j] = fmix64(key[j]) & t.mask;
         }
     }
-    for (uint64_t it = 0; it <= t.mask; ++it) {
-        uint64_t k[R];
+    // two loops, so that the usual few probes carry no test of the error word
+    // (60M rows into 15M hashed groups: 2.93 ms with one loop, 2.89 this way)
+#pragma unroll 1
+    for (uint32_t far = 0; far < AGG_MAX_PROBES; far += AGG_PROBE_STEP) {
+        if (far != 0 && agg_overflowed(err)) return;
+#pragma unroll 1
+        for (uint32_t it = 0; it < AGG_PROBE_STEP; ++it) {
+            uint64_t k[R];
 #pragma unroll
-        for (int j = 0; j < R; ++j)
-            if (act[j]) k[j] = __ldcg((const unsigned long long*)(t.slots + s[j] * t.words));
-        unsigned long long prev[R];
-        bool cas[R];
+            for (int j = 0; j < R; ++j)
+                if (act[j]) k[j] = __ldcg((const unsigned long long*)(t.slots + s[j] * t.words));
+            unsigned long long prev[R];
+            bool cas[R];
 #pragma unroll
-        for (int j = 0; j < R; ++j) {
-            cas[j] = act[j] && k[j] == EMPTY64;
-            if (cas[j])
-                prev[j] = atomicCAS((unsigned long long*)(t.slots + s[j] * t.words), (unsigned long long)EMPTY64,
-                                    (unsigned long long)key[j]);
-        }
-        bool any = false;
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            if (!act[j]) continue;
-            const bool mine = cas[j] ? (prev[j] == EMPTY64 || prev[j] == key[j]) : k[j] == key[j];
-            if (mine) {
-                slot[j] = t.slots + s[j] * t.words;
-                claimed[j] = cas[j] && prev[j] == EMPTY64;
-                act[j] = false;
-            } else {
-                s[j] = (s[j] + 1) & t.mask;
-                any = true;
+            for (int j = 0; j < R; ++j) {
+                cas[j] = act[j] && k[j] == EMPTY64;
+                if (cas[j])
+                    prev[j] = atomicCAS((unsigned long long*)(t.slots + s[j] * t.words), (unsigned long long)EMPTY64,
+                                        (unsigned long long)key[j]);
             }
+            bool any = false;
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                if (!act[j]) continue;
+                const bool mine = cas[j] ? (prev[j] == EMPTY64 || prev[j] == key[j]) : k[j] == key[j];
+                if (mine) {
+                    slot[j] = t.slots + s[j] * t.words;
+                    claimed[j] = cas[j] && prev[j] == EMPTY64;
+                    act[j] = false;
+                } else {
+                    s[j] = (s[j] + 1) & t.mask;
+                    any = true;
+                }
+            }
+            if (!any) return;
         }
-        if (!any) return;
     }
 #pragma unroll
     for (int j = 0; j < R; ++j)

@@ -687,12 +687,22 @@ __device__ __forceinline__ void build_insert(const BuildDev& b, uint64_t i) {
 // claimed is set when this call took a fresh slot.  Callers count their
 // claims and add them to t.used in bulk (agg_add_claims): one counter word
 // updated once per new key by every thread would serialise at its L2 slice.
-// A table that fills up ends the probe with ERR_OVERFLOW.
+// A table that fills up ends the probe with ERR_OVERFLOW: after AGG_MAX_PROBES
+// slots (at 0.9 full, where the execution is retried in any case, the longest
+// run of taken slots expected among 2^27 is about 3,500), or soon after another
+// row has met that.  Walking the whole table, each row of 4M keys too many for
+// a million slots took a million dependent loads: one launch of some 20 s.
+constexpr uint32_t AGG_MAX_PROBES = 16384;
+constexpr uint32_t AGG_PROBE_STEP = 256;   // slots between two looks at the error word
+__device__ __forceinline__ bool agg_overflowed(const uint32_t* err) {
+    return (*(const volatile uint32_t*)err & ERR_OVERFLOW) != 0;
+}
+
 __device__ __forceinline__ uint64_t* agg_slot(const AggTable& t, uint64_t key, uint32_t* err, bool& claimed) {
     claimed = false;
     if (key == EMPTY64) return t.slots + (t.mask + 1) * t.words;   // side slot
     uint64_t s = fmix64(key) & t.mask;
-    for (uint64_t it = 0; it <= t.mask; ++it) {
+    for (uint32_t it = 0; it < AGG_MAX_PROBES; ++it) {
         uint64_t* p = t.slots + s * t.words;
         uint64_t k = __ldcg((const unsigned long long*)p);
         if (k == key) return p;
@@ -706,6 +716,7 @@ __device__ __forceinline__ uint64_t* agg_slot(const AggTable& t, uint64_t key, u
             if (prev == key) return p;
         }
         s = (s + 1) & t.mask;
+        if ((it + 1) % AGG_PROBE_STEP == 0 && agg_overflowed(err)) return nullptr;
     }
     atomicOr(err, ERR_OVERFLOW);
     return nullptr;
