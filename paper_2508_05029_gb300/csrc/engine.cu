@@ -63,7 +63,7 @@ static void free_arena(Budget& b, Lane* l) {
 // further bytes (all: every one).
 static void trim_arenas(Budget& b, uint64_t excess, bool all = false) {
     for (Lane* l : b.lanes) {
-        if (!l->arena || l->busy) continue;
+        if (l->busy || !l->arena) continue;
         if (!all && b.reserved + excess + idle_arenas(b) <= b.cap && b.arenas <= arena_limit(b)) return;
         free_arena(b, l);
     }
@@ -100,20 +100,23 @@ bool lane_drop_arena(tp_engine* e, Lane* lane) {
 }
 
 void lane_grow_arena(tp_engine* e, Lane* lane, uint64_t want, uint64_t reserved) {
-    std::lock_guard<std::mutex> lk(e->budget.mu);
+    if (want <= lane->arena_bytes) return;
     Budget& b = e->budget;
-    const uint64_t excess = want > reserved ? want - reserved : 0;
-    if (want <= lane->arena_bytes || b.arenas - lane->arena_bytes + want > arena_limit(b) ||
-        b.reserved + excess + idle_arenas(b) > b.cap)
-        return;
-    if (lane->arena) free_arena(b, lane);
-    if (cudaMallocAsync(&lane->arena, want, lane->compute) != cudaSuccess) {
-        cudaGetLastError();
-        lane->arena = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(b.mu);
+        const uint64_t excess = want > reserved ? want - reserved : 0;
+        if (b.arenas - lane->arena_bytes + want > arena_limit(b) || b.reserved + excess + idle_arenas(b) > b.cap) return;
+        if (lane->arena) free_arena(b, lane);
+        b.arenas += want;   // counted first: the allocation may map memory, and nobody waits for that
+    }
+    if (cudaMallocAsync(&lane->arena, want, lane->compute) == cudaSuccess) {
+        lane->arena_bytes = want;
         return;
     }
-    lane->arena_bytes = want;
-    b.arenas += want;
+    cudaGetLastError();
+    lane->arena = nullptr;
+    std::lock_guard<std::mutex> lk(b.mu);
+    b.arenas -= want;
 }
 
 bool lane_over(tp_engine* e, uint64_t excess) {
