@@ -328,15 +328,9 @@ __global__ void k_many_count(const __grid_constant__ BuildDev b, uint64_t n, uin
         }
         const int64_t key = ld1(b.key, i);
         if (b.jt.lip != nullptr) lip_insert(b.jt, key);
-        uint32_t payload = 0;
-        for (int f = 0; f < b.n_dfield; ++f) {
-            const int64_t v = ld1(b.dcol[f], i);
-            if (v < 0 || ((uint64_t)v >> b.dbits[f]) != 0) payload |= PAYLOAD_BAD;
-            else payload |= (uint32_t)((uint64_t)v << b.dpos[f]);
-        }
         uint32_t rank = 0;
         const uint64_t s = many_insert(b.jt, key, b.err, &rank);
-        pays[i] = payload;
+        pays[i] = build_payload(b, i);
         place[i] = s == MANY_NONE ? MANY_NONE : (s << MANY_RANK_BITS) | rank;
     }
 }
